@@ -54,7 +54,7 @@ def listed():
         # the default workload: decaying Mach-2 turbulence on one 256^3 box
         _gas("turb256_fp32", (256, 256, 256), 20, flow="turbulence", gamma=1.0001),
         # the paper's throughput set-up: PLM + HLLE + RK2 on a mesh of linked 128^3 blocks
-        _gas("blocks256_hlle_rk2", (256, 256, 256), 30, riemann="hlle", integrator="rk2", split=2),
+        _gas("blocks256_hlle_rk2", (256, 256, 256), 50, riemann="hlle", integrator="rk2", split=2),
         # a production box whose sizes divide nothing, third-order reconstruction and time steps
         _gas("ragged_ppm_rk3", (190, 131, 77), 20, recon="ppm", integrator="rk3"),
         # the FP64 path that results are validated with
@@ -65,7 +65,7 @@ def listed():
         _gas("vortex128_hydro", (128, 128, 128), 40, flow="vortex", eos="hydro", riemann="lhlld", integrator="rk2"),
         # many independent uneven boxes (16 to 64 cells a side, every third spherical) in one context, with
         # one time step that the program gives
-        {"name": "boxes512_uneven", "kind": "boxes", "blocks": 512, "steps": 10, "gamma": 5.0 / 3.0},
+        {"name": "boxes512_uneven", "kind": "boxes", "blocks": 512, "steps": 20, "gamma": 5.0 / 3.0},
         # gas and eight dust species, the drag solved in FP64
         _dust("dust128_fp64drag", (128, 128, 128), 10, 8, "fp64"),
         # a small ragged dust box, the drag in FP64 only for the stiff species
