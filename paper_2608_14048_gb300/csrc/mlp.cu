@@ -13,8 +13,8 @@
 // accepted if every flux lies within mlp_tau of the HLL dissipation bracket
 // around HLLE plus 2e-2 of its scale.
 //
-// Training runs on the GPU with the project's own FP32 kernels (tiled SGEMM,
-// SiLU backward, Adam).  Inference runs on the tensor cores in BF16 with
+// Training runs on the GPU with the project's own FP32 kernels (row tiles
+// through all layers, split weight gradients, Adam).  Inference runs on the tensor cores in BF16 with
 // FP32 accumulation (mma.sync m16n8k16): a warp pushes 16 faces at a time
 // through all four layers, keeping the hidden activations in registers
 // (each layer's accumulator fragments are exactly the next layer's A
@@ -97,107 +97,390 @@ __global__ void __launch_bounds__(256)
 }
 
 // ------------------------------------------------------------------------
-// FP32 training kernels
+// FP32 training kernels: the gradient of a batch in three launches.
+//
+//   k_mlp_rows   forward and backward of a tile of rows: every layer of a row
+//                depends on that row alone, so a CTA keeps the activations of
+//                its rows in shared memory through all eight products, with
+//                W2 and W3 resident (both directions read the same rows of W);
+//   k_mlp_dw     weight gradients dW_l = dZ_l^T A_(l-1), the sum over the
+//                batch split into chunks so that the chip is full;
+//   k_mlp_dsum   the chunks' sums, in a fixed order.
+//
+// Bound: FP32 FMA issue (6 x 35,840 FMA-flop a row) and the shared-memory
+// wavefronts of the operands.  Packed FP32 FMAs (two a lane and instruction)
+// halve the issue slots.  Before, eleven tiled products (64 x 64 tiles: four
+// CTAs over K = batch for a weight gradient) and fourteen elementwise passes:
+// 3524 us for a batch of 8192 with
+// Adam, 88 us now (15.8 TFLOP/s over the whole call's five launches); the
+// error of the gradient against FP64 fell from 1.1e-6 to 9e-8.
 // ------------------------------------------------------------------------
-// C[m][n] = alpha * sum_k A(m,k) B(k,n) + beta * C[m][n]; A(m,k) = A[m*sam + k*sak],
-// B(k,n) = B[k*sbk + n*sbn], C row-major with ldc.  64x64 tiles, 256 threads.
-__global__ void __launch_bounds__(256)
-    k_sgemm(int M, int N, int K, float alpha, const float* __restrict__ A, long long sam,
-            long long sak, const float* __restrict__ B, long long sbk, long long sbn, float beta,
-            float* __restrict__ C, long long ldc) {
-  __shared__ float As[16][64 + 4];
-  __shared__ float Bs[16][64 + 4];
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-  float acc[4][4] = {};
-  for (int k0 = 0; k0 < K; k0 += 16) {
-    for (int e = threadIdx.x; e < 16 * 64; e += 256) {
-      const int kk = e / 64, mm = e % 64;
-      const int gm = m0 + mm, gk = k0 + kk;
-      As[kk][mm] = (gm < M && gk < K) ? A[gm * sam + gk * sak] : 0.0f;
-      const int gn = n0 + mm;
-      Bs[kk][mm] = (gn < N && gk < K) ? B[gk * sbk + gn * sbn] : 0.0f;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < 16; ++kk) {
-      float a[4], b[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) { a[q] = As[kk][ty * 4 + q]; b[q] = Bs[kk][tx * 4 + q]; }
-#pragma unroll
-      for (int p = 0; p < 4; ++p)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) acc[p][q] += a[p] * b[q];
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int p = 0; p < 4; ++p)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int gm = m0 + ty * 4 + p, gn = n0 + tx * 4 + q;
-      if (gm < M && gn < N) {
-        float v = alpha * acc[p][q];
-        if (beta != 0.0f) v += beta * C[gm * ldc + gn];
-        C[gm * ldc + gn] = v;
-      }
-    }
-}
-
 __device__ __forceinline__ float silu_f(float z) { return z / (1.0f + __expf(-z)); }
 __device__ __forceinline__ float dsilu_f(float z) {
   const float s = 1.0f / (1.0f + __expf(-z));
   return s * (1.0f + z * (1.0f - s));
 }
 
-// Z[s][o] += b[o]; A = silu(Z) (or A = Z for the output layer)
-__global__ void k_bias_act(float* __restrict__ Z, float* __restrict__ Aout, const float* __restrict__ b,
-                           int n, int width, int ld, int act) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (long long)n * width) return;
-  const int s = (int)(t / width), o = (int)(t % width);
-  const float z = Z[(long long)s * ld + o] + b[o];
-  Z[(long long)s * ld + o] = z;
-  Aout[(long long)s * ld + o] = act ? silu_f(z) : z;
-}
+// c += a * b on both halves
+__device__ __forceinline__ void fma2(float2& c, float2 a, float2 b) { c = __ffma2_rn(a, b, c); }
 
-// dY = (Yhat - Y) / n over the 7 real outputs; loss partial sums
-__global__ void k_loss(const float* __restrict__ Yh, const float* __restrict__ Y, float* __restrict__ dY,
-                       int n, float* __restrict__ loss) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  float l = 0.0f;
-  if (s < n) {
-    for (int o = 0; o < MLP_OUT; ++o) {
-      const float e = Yh[(long long)s * MLP_OUTP + o] - Y[(long long)s * MLP_OUTP + o];
-      dY[(long long)s * MLP_OUTP + o] = e / n;
-      l += 0.5f * e * e;
+__device__ __forceinline__ void cp4(float* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(
+                   static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
+               "l"(src));
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
+
+// Shared memory of k_mlp_rows (floats).  Row pitches of 132 and 20: eight
+// lanes that read 16 bytes of eight consecutive rows touch all 32 banks.
+constexpr int RW_LD = 132, RW_LD1 = 20;
+template <int TM>
+struct RowsSmem {
+  float w2[128 * RW_LD], w3[128 * RW_LD], w1[128 * RW_LD1], w4[MLP_OUT * RW_LD];
+  float a[8 * TM * RW_LD];        // activations of the tile's rows, then their gradients
+  float x[8 * TM * RW_LD1];       // inputs, columns 14.. zero
+  float dy[8 * TM * MLP_OUTP];
+  float b[3 * 128 + MLP_OUTP];
+  float red[8];
+};
+
+// acc[r][j] = sum_k A[m][k] B[n][k]: rows m = TM warp + r, columns n = lane + 32 j.
+// The two halves of an accumulator take the even and the odd k, so that both
+// operands are read as they lie.
+template <int TM, int K, int LD>
+__device__ __forceinline__ void rows_nt(const float* A, const float* B, float (&out)[TM][4]) {
+  const int lane = threadIdx.x & 31, m0 = TM * (threadIdx.x >> 5);
+  float2 acc[TM][4];
+#pragma unroll
+  for (int r = 0; r < TM; ++r)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[r][j] = make_float2(0.0f, 0.0f);
+#pragma unroll 4
+  for (int k = 0; k < K; k += 4) {
+    float4 b[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) b[j] = *reinterpret_cast<const float4*>(B + (lane + 32 * j) * LD + k);
+#pragma unroll
+    for (int r = 0; r < TM; ++r) {
+      const float4 a = *reinterpret_cast<const float4*>(A + (m0 + r) * LD + k);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        fma2(acc[r][j], make_float2(a.x, a.y), make_float2(b[j].x, b[j].y));
+        fma2(acc[r][j], make_float2(a.z, a.w), make_float2(b[j].z, b[j].w));
+      }
     }
-    dY[(long long)s * MLP_OUTP + 7] = 0.0f;
   }
-  for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-  if ((threadIdx.x & 31) == 0) atomicAdd(loss, l / n);
+#pragma unroll
+  for (int r = 0; r < TM; ++r)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) out[r][j] = acc[r][j].x + acc[r][j].y;
 }
 
-// db[o] = sum_s dZ[s][o]
-__global__ void k_colsum(const float* __restrict__ dZ, float* __restrict__ db, int n, int width, int ld) {
-  const int o = blockIdx.x;
-  float acc = 0.0f;
-  for (int s = threadIdx.x; s < n; s += blockDim.x) acc += dZ[(long long)s * ld + o];
-  for (int q = 16; q > 0; q >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, q);
-  __shared__ float sm[32];
-  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = acc;
+// out[r][j] = sum_k A[m][k] B[k][n]: rows as above, columns n = 4 lane + j.
+template <int TM>
+__device__ __forceinline__ void rows_nn(const float* A, const float* B, float (&out)[TM][4]) {
+  const int lane = threadIdx.x & 31, m0 = TM * (threadIdx.x >> 5);
+  float2 acc[TM][2];
+#pragma unroll
+  for (int r = 0; r < TM; ++r) acc[r][0] = acc[r][1] = make_float2(0.0f, 0.0f);
+#pragma unroll 2
+  for (int k = 0; k < 128; k += 4) {
+    float4 b[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) b[q] = *reinterpret_cast<const float4*>(B + (k + q) * RW_LD + 4 * lane);
+#pragma unroll
+    for (int r = 0; r < TM; ++r) {
+      const float4 a = *reinterpret_cast<const float4*>(A + (m0 + r) * RW_LD + k);
+      const float av[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        fma2(acc[r][0], make_float2(av[q], av[q]), make_float2(b[q].x, b[q].y));
+        fma2(acc[r][1], make_float2(av[q], av[q]), make_float2(b[q].z, b[q].w));
+      }
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < TM; ++r) {
+    out[r][0] = acc[r][0].x; out[r][1] = acc[r][0].y;
+    out[r][2] = acc[r][1].x; out[r][3] = acc[r][1].y;
+  }
+}
+
+// Forward and backward of the rows, tiles of 8 TM rows (TM a warp) per
+// iteration of a persistent CTA.  Act[l]: activations of hidden layer l + 1;
+// dZ[l]: silu'(Z) on the way forward, then the gradient of Z; dY: gradient
+// of the outputs; all row-major in global memory for k_mlp_dw.
+struct RowsOut {
+  float* act[3];
+  float* dz[3];
+  float* dy;
+};
+
+template <int TM>
+__global__ void __launch_bounds__(256, 1)
+    k_mlp_rows(const float* __restrict__ params, const float* __restrict__ X,
+               const float* __restrict__ Y, int n, RowsOut o, float* __restrict__ loss) {
+  extern __shared__ __align__(16) unsigned char rows_smem[];
+  RowsSmem<TM>& S = *reinterpret_cast<RowsSmem<TM>*>(rows_smem);
+  constexpr int TR = 8 * TM;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, m0 = TM * warp;
+  const float* W1 = params;
+  const float* W2 = W1 + 128 * MLP_IN + 128;
+  const float* W3 = W2 + 128 * 128 + 128;
+  const float* W4 = W3 + 128 * 128 + 128;
+  auto load_x = [&](long long row0) {
+    for (int e = tid; e < TR * MLP_IN; e += 256) {
+      const int r = e / MLP_IN, c = e % MLP_IN;
+      if (row0 + r < n) cp4(S.x + r * RW_LD1 + c, X + (row0 + r) * MLP_INP + c);
+      else S.x[r * RW_LD1 + c] = 0.0f;
+    }
+  };
+  // weights: the first layer's operands, then W2, then W3 (three groups)
+  for (int e = tid; e < 128 * MLP_IN; e += 256) cp4(S.w1 + (e / MLP_IN) * RW_LD1 + e % MLP_IN, W1 + e);
+  for (int e = tid; e < 128 * 6; e += 256) S.w1[(e / 6) * RW_LD1 + MLP_IN + e % 6] = 0.0f;
+  for (int e = tid; e < TR * 6; e += 256) S.x[(e / 6) * RW_LD1 + MLP_IN + e % 6] = 0.0f;
+  for (int e = tid; e < MLP_OUT * 128; e += 256) cp4(S.w4 + (e / 128) * RW_LD + e % 128, W4 + e);
+  if (tid < 128) {
+    S.b[tid] = W2[tid - 128];
+    S.b[128 + tid] = W3[tid - 128];
+    S.b[256 + tid] = W4[tid - 128];
+  } else if (tid < 128 + MLP_OUT) {
+    S.b[384 + tid - 128] = W4[MLP_OUT * 128 + tid - 128];
+  }
+  load_x((long long)blockIdx.x * TR);
+  cp_commit();
+  for (int e = tid; e < 128 * 128; e += 256) cp4(S.w2 + (e / 128) * RW_LD + e % 128, W2 + e);
+  cp_commit();
+  for (int e = tid; e < 128 * 128; e += 256) cp4(S.w3 + (e / 128) * RW_LD + e % 128, W3 + e);
+  cp_commit();
+  float lsum = 0.0f;
+  bool first = true;
+  for (long long row0 = (long long)blockIdx.x * TR; row0 < n; row0 += (long long)gridDim.x * TR) {
+    float acc[TM][4];
+    if (first) cp_wait<2>();
+    else cp_wait<0>();
+    __syncthreads();
+    // hidden layer l from the product in acc (columns lane + 32 j)
+    auto hidden = [&](int l) {
+#pragma unroll
+      for (int r = 0; r < TM; ++r)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int c = lane + 32 * j;
+          const float z = acc[r][j] + S.b[128 * l + c];
+          const float a = silu_f(z);
+          S.a[(m0 + r) * RW_LD + c] = a;
+          if (row0 + m0 + r < n) {
+            o.act[l][(row0 + m0 + r) * 128 + c] = a;
+            o.dz[l][(row0 + m0 + r) * 128 + c] = dsilu_f(z);
+          }
+        }
+    };
+    rows_nt<TM, 16, RW_LD1>(S.x, S.w1, acc);
+    hidden(0);
+    if (first) cp_wait<1>();
+    __syncthreads();
+    rows_nt<TM, 128, RW_LD>(S.a, S.w2, acc);
+    __syncwarp();   // a warp reads and writes its own rows of S.a only
+    hidden(1);
+    if (first) cp_wait<0>();
+    __syncthreads();
+    rows_nt<TM, 128, RW_LD>(S.a, S.w3, acc);
+    __syncwarp();
+    hidden(2);
+    __syncwarp();
+    // output layer and its gradient (yhat - y) / n: the warp's TM rows
+    for (int e = lane; e < TM * MLP_OUTP; e += 32) {
+      const int r = m0 + e / MLP_OUTP, q = e % MLP_OUTP;
+      float g = 0.0f;
+      if (q < MLP_OUT && row0 + r < n) {
+        float2 s = make_float2(0.0f, 0.0f);
+#pragma unroll 8
+        for (int k = 0; k < 128; k += 4) {
+          const float4 a = *reinterpret_cast<const float4*>(S.a + r * RW_LD + k);
+          const float4 w = *reinterpret_cast<const float4*>(S.w4 + q * RW_LD + k);
+          fma2(s, make_float2(a.x, a.y), make_float2(w.x, w.y));
+          fma2(s, make_float2(a.z, a.w), make_float2(w.z, w.w));
+        }
+        const float d = s.x + s.y + S.b[384 + q] - Y[(row0 + r) * MLP_OUTP + q];
+        g = d / n;
+        lsum += 0.5f * d * d;
+      }
+      S.dy[r * MLP_OUTP + q] = g;
+      if (row0 + r < n) o.dy[(row0 + r) * MLP_OUTP + q] = g;
+    }
+    __syncwarp();
+    // dZ of hidden layer l from the product in acc (columns 4 lane + j); the
+    // silu' values were written by this CTA's other lanes before a barrier
+    auto back = [&](int l) {
+#pragma unroll
+      for (int r = 0; r < TM; ++r)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int c = 4 * lane + j;
+          float g = 0.0f;
+          if (row0 + m0 + r < n) {
+            float* p = o.dz[l] + (row0 + m0 + r) * 128 + c;
+            g = acc[r][j] * *p;
+            *p = g;
+          }
+          S.a[(m0 + r) * RW_LD + c] = g;
+        }
+    };
+#pragma unroll
+    for (int r = 0; r < TM; ++r) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[r][j] = 0.0f;
+#pragma unroll
+      for (int q = 0; q < MLP_OUT; ++q) {
+        const float g = S.dy[(m0 + r) * MLP_OUTP + q];
+        const float4 w = *reinterpret_cast<const float4*>(S.w4 + q * RW_LD + 4 * lane);
+        acc[r][0] += g * w.x; acc[r][1] += g * w.y; acc[r][2] += g * w.z; acc[r][3] += g * w.w;
+      }
+    }
+    back(2);
+    __syncwarp();
+    rows_nn<TM>(S.a, S.w3, acc);
+    __syncwarp();
+    back(1);
+    __syncwarp();
+    rows_nn<TM>(S.a, S.w2, acc);
+    __syncwarp();
+    back(0);
+    __syncthreads();
+    first = false;
+    load_x(row0 + (long long)gridDim.x * TR);
+    cp_commit();
+  }
+  cp_wait<0>();
+  for (int q = 16; q > 0; q >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, q);
+  if (lane == 0) S.red[warp] = lsum;
   __syncthreads();
-  if (threadIdx.x < 32) {
-    float v = threadIdx.x < (blockDim.x >> 5) ? sm[threadIdx.x] : 0.0f;
-    for (int q = 16; q > 0; q >>= 1) v += __shfl_xor_sync(0xffffffffu, v, q);
-    if (threadIdx.x == 0) db[o] = v;
+  if (tid == 0) {
+    float l = 0.0f;
+    for (int w = 0; w < 8; ++w) l += S.red[w];
+    if (l != 0.0f) atomicAdd(loss, l / n);   // a NaN compares unequal and is added
   }
 }
 
-// dZ = dA * silu'(Z)
-__global__ void k_dsilu(float* __restrict__ dA, const float* __restrict__ Z, long long n) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < n) dA[t] *= dsilu_f(Z[t]);
+// Weight and bias gradients of the rows [chunk * rows, ...): blockIdx.x = 0, 1
+// the 128 x 128 layers 2 and 3 (8 x 8 outputs a thread), 2 the thin layers 1
+// and 4.  Row-major results at part + chunk * MLP_NPARAM.
+constexpr int DW_K = 16;   // rows staged at a time
+
+__global__ void __launch_bounds__(256, 2)
+    k_mlp_dw(const float* __restrict__ X, RowsOut o, int n, int rows, float* __restrict__ part) {
+  const long long r0 = (long long)blockIdx.y * rows, r1 = min((long long)n, r0 + rows);
+  part += (long long)blockIdx.y * MLP_NPARAM;
+  const int tid = threadIdx.x;
+  constexpr int OFF2 = 128 * MLP_IN + 128, OFF3 = OFF2 + 128 * 129, OFF4 = OFF3 + 128 * 129;
+  if (blockIdx.x == 2) {
+    // layer 1: thread (o, half) takes 7 inputs; layer 4: thread (i, half) 4
+    // outputs (3 in the upper half)
+    const int c = tid & 127, half = tid >> 7;
+    float g1[7] = {}, gb1 = 0.0f, g4[4] = {}, gb4 = 0.0f;
+#pragma unroll 4
+    for (long long s = r0; s < r1; ++s) {
+      const float d = o.dz[0][s * 128 + c], a = o.act[2][s * 128 + c];
+#pragma unroll
+      for (int q = 0; q < 7; ++q) g1[q] += d * X[s * MLP_INP + 7 * half + q];
+      gb1 += d;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) g4[q] += a * o.dy[s * MLP_OUTP + 4 * half + q];
+      if (tid < MLP_OUT) gb4 += o.dy[s * MLP_OUTP + tid];
+    }
+#pragma unroll
+    for (int q = 0; q < 7; ++q) part[c * MLP_IN + 7 * half + q] = g1[q];
+    if (half == 0) part[128 * MLP_IN + c] = gb1;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (4 * half + q < MLP_OUT) part[OFF4 + (4 * half + q) * 128 + c] = g4[q];
+    if (tid < MLP_OUT) part[OFF4 + MLP_OUT * 128 + tid] = gb4;
+    return;
+  }
+  const int l = 1 + blockIdx.x;   // gradient of hidden layer l + 1
+  const float* __restrict__ D = l == 1 ? o.dz[1] : o.dz[2];
+  const float* __restrict__ A = l == 1 ? o.act[0] : o.act[1];
+  __shared__ __align__(16) float sD[2][DW_K][128], sA[2][DW_K][128];
+  const int tx = tid & 15, ty = tid >> 4;
+  float2 acc[8][4];
+  float gb = 0.0f;
+#pragma unroll
+  for (int p = 0; p < 8; ++p)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[p][q] = make_float2(0.0f, 0.0f);
+  auto stage = [&](long long s0, int buf) {
+#pragma unroll
+    for (int e = 0; e < DW_K * 128; e += 256) {
+      const int r = (e + tid) >> 7, c = tid & 127;
+      if (s0 + r < r1) {
+        cp4(&sD[buf][r][c], D + (s0 + r) * 128 + c);
+        cp4(&sA[buf][r][c], A + (s0 + r) * 128 + c);
+      } else {
+        sD[buf][r][c] = 0.0f;
+        sA[buf][r][c] = 0.0f;
+      }
+    }
+    cp_commit();
+  };
+  stage(r0, 0);
+  int buf = 0;
+  for (long long s0 = r0; s0 < r1; s0 += DW_K, buf ^= 1) {
+    if (s0 + DW_K < r1) {
+      stage(s0 + DW_K, buf ^ 1);
+      cp_wait<1>();
+    } else {
+      cp_wait<0>();
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int k = 0; k < DW_K; ++k) {
+      const float4 a0 = *reinterpret_cast<const float4*>(&sD[buf][k][4 * ty]);
+      const float4 a1 = *reinterpret_cast<const float4*>(&sD[buf][k][64 + 4 * ty]);
+      const float4 b0 = *reinterpret_cast<const float4*>(&sA[buf][k][4 * tx]);
+      const float4 b1 = *reinterpret_cast<const float4*>(&sA[buf][k][64 + 4 * tx]);
+      const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+      const float2 b[4] = {make_float2(b0.x, b0.y), make_float2(b0.z, b0.w), make_float2(b1.x, b1.y),
+                           make_float2(b1.z, b1.w)};
+#pragma unroll
+      for (int p = 0; p < 8; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) fma2(acc[p][q], make_float2(a[p], a[p]), b[q]);
+    }
+    if (tid < 128) {
+#pragma unroll
+      for (int k = 0; k < DW_K; ++k) gb += sD[buf][k][tid];
+    }
+    __syncthreads();
+  }
+  float* __restrict__ out = part + (l == 1 ? OFF2 : OFF3);
+#pragma unroll
+  for (int p = 0; p < 8; ++p)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int m = (p < 4 ? 0 : 60) + 4 * ty + p, c = (q < 2 ? 0 : 60) + 4 * tx + 2 * q;
+      out[m * 128 + c] = acc[p][q].x;
+      out[m * 128 + c + 1] = acc[p][q].y;
+    }
+  if (tid < 128) out[128 * 128 + tid] = gb;
+}
+
+// grad = sum of the chunks' gradients: four groups of chunks a parameter, in
+// a fixed order
+__global__ void __launch_bounds__(256) k_mlp_dsum(const float* __restrict__ part, int chunks,
+                                                  float* __restrict__ grad) {
+  __shared__ float sm[4][64];
+  const int c = threadIdx.x & 63, g = threadIdx.x >> 6;
+  const long long p = (long long)blockIdx.x * 64 + c;
+  float acc = 0.0f;
+  if (p < MLP_NPARAM)
+#pragma unroll 4
+    for (int q = g; q < chunks; q += 4) acc += part[(long long)q * MLP_NPARAM + p];
+  sm[g][c] = acc;
+  __syncthreads();
+  if (g == 0 && p < MLP_NPARAM) grad[p] = (sm[0][c] + sm[1][c]) + (sm[2][c] + sm[3][c]);
 }
 
 __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
@@ -211,13 +494,6 @@ __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float
   m[t] = mt;
   v[t] = vt;
   p[t] -= lr * (mt / c1) / (sqrtf(vt / c2) + eps);
-}
-
-static void sgemm(cudaStream_t st, int M, int N, int K, float alpha, const float* A, long long sam,
-                  long long sak, const float* B, long long sbk, long long sbn, float beta, float* C,
-                  long long ldc) {
-  dim3 grd((N + 63) / 64, (M + 63) / 64);
-  k_sgemm<<<grd, 256, 0, st>>>(M, N, K, alpha, A, sam, sak, B, sbk, sbn, beta, C, ldc);
 }
 
 // Parameter offsets of the unpadded layout (per layer: W[out][in], b[out]).
@@ -246,60 +522,50 @@ extern "C" aeth_status aeth_mlp_grad(const float* d_params, const float* d_X, co
   aeth_mlp_work_floats(n, &need);
   if (work_floats < need) return AETH_ERR_ARG;
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  long long off[5];
-  layer_offsets(off);
-  const int dims[5] = {MLP_IN, MLP_H, MLP_H, MLP_H, MLP_OUT};
   const long long H = MLP_H;
-  float* Z[4];
-  float* Aact[4];
+  RowsOut o;
   float* w = d_work;
-  for (int l = 1; l <= 3; ++l) { Z[l] = w; w += (long long)n * H; Aact[l] = w; w += (long long)n * H; }
-  float* Yh = w; w += (long long)n * MLP_OUTP;
-  float* dY = w; w += (long long)n * MLP_OUTP;
-  float* dZa = w; w += (long long)n * H;
-  float* dZb = w;
-  const int T = 256;
-  // forward: Z_l = A_{l-1} W_l^T, + b, act
-  const float* prev = d_X;
-  long long ldp = MLP_INP;
-  for (int l = 0; l < 4; ++l) {
-    const int nin = dims[l], nout = dims[l + 1];
-    const float* W = d_params + off[l];
-    const float* b = W + (long long)nout * nin;
-    float* Zo = l < 3 ? Z[l + 1] : Yh;
-    float* Ao = l < 3 ? Aact[l + 1] : Yh;
-    const long long ldo = l < 3 ? H : MLP_OUTP;
-    sgemm(st, n, nout, nin, 1.0f, prev, ldp, 1, W, 1, nin, 0.0f, Zo, ldo);
-    k_bias_act<<<(int)(((long long)n * nout + T - 1) / T), T, 0, st>>>(Zo, Ao, b, n, nout, (int)ldo, l < 3);
-    prev = Ao;
-    ldp = ldo;
-  }
+  for (int l = 0; l < 3; ++l) { o.act[l] = w; w += (long long)n * H; }
+  for (int l = 0; l < 3; ++l) { o.dz[l] = w; w += (long long)n * H; }
+  o.dy = w;
+  w += (long long)n * MLP_OUTP;
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return AETH_ERR_CUDA;
   if (cudaMemsetAsync(d_loss, 0, sizeof(float), st) != cudaSuccess) return AETH_ERR_CUDA;
-  k_loss<<<(n + T - 1) / T, T, 0, st>>>(Yh, d_Y, dY, n, d_loss);
-  // backward
-  const float* dZ = dY;
-  long long ldz = MLP_OUTP;
-  float* bufs[2] = {dZa, dZb};
-  for (int l = 3; l >= 0; --l) {
-    const int nin = dims[l], nout = dims[l + 1];
-    const float* W = d_params + off[l];
-    float* gW = d_grad + off[l];
-    float* gb = gW + (long long)nout * nin;
-    const float* Ain = l > 0 ? Aact[l] : d_X;
-    const long long lda = l > 0 ? H : MLP_INP;
-    // dW = dZ^T A_in : M = nout, N = nin, K = n
-    sgemm(st, nout, nin, n, 1.0f, dZ, 1, ldz, Ain, lda, 1, 0.0f, gW, nin);
-    k_colsum<<<nout, 256, 0, st>>>(dZ, gb, n, nout, (int)ldz);
-    if (l > 0) {
-      float* dA = bufs[l & 1];
-      // dA = dZ W : M = n, N = nin, K = nout
-      sgemm(st, n, nin, nout, 1.0f, dZ, ldz, 1, W, nin, 1, 0.0f, dA, H);
-      const long long tot = (long long)n * H;
-      k_dsilu<<<(int)((tot + T - 1) / T), T, 0, st>>>(dA, Z[l], tot);
-      dZ = dA;
-      ldz = H;
-    }
+  // rows a tile: the TM (rows a warp) with the fewest row-rounds of the
+  // chip, a round costing its rows plus about two rows of fixed work
+  auto rows = [&](auto kernel, int tm, size_t smem) -> bool {
+    const int tiles = ceil_div(n, 8 * tm);
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+      return false;
+    kernel<<<std::min(tiles, sms), 256, smem, st>>>(d_params, d_X, d_Y, n, o, d_loss);
+    return true;
+  };
+  int tm = 8;
+  long long best = -1;
+  for (int t : {8, 7, 4, 2}) {
+    const long long cost = (long long)ceil_div(ceil_div(n, 8 * t), sms) * (t + 2);
+    if (best < 0 || cost < best) { best = cost; tm = t; }
   }
+  const bool ok = tm == 8   ? rows(k_mlp_rows<8>, 8, sizeof(RowsSmem<8>))
+                  : tm == 7 ? rows(k_mlp_rows<7>, 7, sizeof(RowsSmem<7>))
+                  : tm == 4 ? rows(k_mlp_rows<4>, 4, sizeof(RowsSmem<4>))
+                            : rows(k_mlp_rows<2>, 2, sizeof(RowsSmem<2>));
+  if (!ok) return AETH_ERR_CUDA;
+  // chunks of the batch for the weight gradients: as many as the rest of the
+  // workspace holds (one per 133 rows) and up to two CTAs an SM; a single
+  // chunk writes the gradient itself
+  const long long room = (d_work + need - w) / MLP_NPARAM;
+  int chunks = (int)std::max(
+      1LL, std::min(room, std::min(2LL * sms / 3, (long long)ceil_div(n, 2 * DW_K))));
+  const int per = ceil_div(ceil_div(n, chunks), DW_K) * DW_K;
+  chunks = ceil_div(n, per);
+  float* part = chunks > 1 ? w : d_grad;
+  k_mlp_dw<<<dim3(3, chunks), 256, 0, st>>>(d_X, o, n, per, part);
+  if (chunks > 1)
+    k_mlp_dsum<<<ceil_div(MLP_NPARAM, 64), 256, 0, st>>>(part, chunks, d_grad);
   return cudaGetLastError() == cudaSuccess ? AETH_OK : AETH_ERR_CUDA;
 }
 
