@@ -12,6 +12,7 @@
 // The kernel template lives here so that its instantiations (one per
 // Riemann solver family) compile in separate translation units.
 #pragma once
+#include "riemann2.cuh"
 #include "runtime.hpp"
 #include "stage.cuh"
 
@@ -41,6 +42,12 @@ __host__ __device__ constexpr int flux_minb(int txt) {
                   : (sizeof(R) == 4 ? (RECON >= 2 ? AETH_FLUX_MINB_2D_PPM : AETH_FLUX_MINB_2D) : 2);
 }
 
+// a compile-time direction as an argument
+template <int V>
+struct Int {
+  static constexpr int value = V;
+};
+
 __host__ __device__ __forceinline__ int ceil_div_d(int a, int b) { return (a + b - 1) / b; }
 
 // Shared-memory plane (one variable, tile + halo) of a band tile (TXT = 0,
@@ -55,11 +62,14 @@ __host__ __device__ constexpr int band_smem(int halo) {
   return m;
 }
 
-// Values of one staged variable plane of a flux tile TXT wide (0: band).
+// Cells of one staged plane of a flux tile TXT wide (0: band), rounded up to
+// a multiple of 4 so that every plane of quads starts on a 16-byte boundary
+// whatever the number of words staged per cell.
 template <int RECON>
 __host__ __device__ constexpr int flux_plane(int txt) {
-  return txt ? (txt + 2 * recon_reach<RECON>() + 1) * (FLUX_NT / txt + 2 * recon_reach<RECON>() + 1)
-             : band_smem(2 * recon_reach<RECON>() + 1);
+  const int n = txt ? (txt + 2 * recon_reach<RECON>() + 1) * (FLUX_NT / txt + 2 * recon_reach<RECON>() + 1)
+                    : band_smem(2 * recon_reach<RECON>() + 1);
+  return (n + 3) / 4 * 4;
 }
 
 // Planes in the shared-memory ring of a 2-D flux tile: the z-queue takes
@@ -74,19 +84,102 @@ __host__ __device__ constexpr int flux_ring(int txt) { return txt ? recon_reach<
 // Solver families 3 and 4 are the isothermal ones.
 constexpr bool iso_solver(int solver) { return solver == 3 || solver == 4; }
 
-// Riemann solver family SOLVER (numbering of k_flux3 below) on one face.
-template <int SOLVER, typename R>
-__device__ __forceinline__ void solve_face(R g, const R* wl, const R* wr, R bn, R* fx) {
+// Riemann solver family SOLVER (numbering of k_flux3 below) on one face, the
+// states as 7 values a side (FP64) or as packed pairs (FP32).
+template <int SOLVER, bool MHD>
+__device__ __forceinline__ void solve_face(double g, double, const double* wl, const double* wr,
+                                           double bn, double* fx) {
   if constexpr (SOLVER == 2) hlle(g, wl, wr, bn, fx);
   else if constexpr (SOLVER == 3) hlld_iso(g, wl, wr, bn, fx);
   else if constexpr (SOLVER == 4) hlle_iso(g, wl, wr, bn, fx);
   else if constexpr (SOLVER == 5) hlld<true>(g, wl, wr, bn, fx);
   else hlld(g, wl, wr, bn, fx);
 }
+template <int SOLVER, bool MHD>
+__device__ __forceinline__ void solve_face(float g, float igm1, const float* wl, const float* wr,
+                                           float bn, float* fx) {
+  float2 W[7];
+#pragma unroll
+  for (int v = 0; v < 7; ++v) W[v] = make_float2(wl[v], wr[v]);
+  if constexpr (SOLVER == 2) hlle2<MHD, false>(g, igm1, W, bn, fx);
+  else if constexpr (SOLVER == 3) hlld_iso2<MHD>(g * g, W, bn, fx);
+  else if constexpr (SOLVER == 4) hlle2<MHD, true>(g * g, igm1, W, bn, fx);
+  else if constexpr (SOLVER == 5) hlld2<true, MHD>(g, igm1, W, bn, fx);
+  else hlld2<false, MHD>(g, igm1, W, bn, fx);
+}
+
+// Four staged values of a cell (16-byte shared accesses in FP32).
+template <typename R>
+struct Quad {
+  R v[4];
+};
+__device__ __forceinline__ Quad<float> ld_quad(const float* p) {
+  const float4 t = *reinterpret_cast<const float4*>(p);
+  return {{t.x, t.y, t.z, t.w}};
+}
+__device__ __forceinline__ Quad<double> ld_quad(const double* p) {
+  const double2 a = *reinterpret_cast<const double2*>(p), b = *reinterpret_cast<const double2*>(p + 2);
+  return {{a.x, a.y, b.x, b.y}};
+}
+__device__ __forceinline__ void st_quad(float* p, float a, float b, float c, float d) {
+  *reinterpret_cast<float4*>(p) = make_float4(a, b, c, d);
+}
+__device__ __forceinline__ void st_quad(double* p, double a, double b, double c, double d) {
+  *reinterpret_cast<double2*>(p) = make_double2(a, b);
+  *reinterpret_cast<double2*>(p + 2) = make_double2(c, d);
+}
+
+// Half the van Leer slopes of four variables of a cell (PLM).
+__device__ __forceinline__ Quad<float> plm_half(const Quad<float>& m, const Quad<float>& c,
+                                                const Quad<float>& p) {
+  Quad<float> t;
+#pragma unroll
+  for (int q = 0; q < 4; q += 2) {
+    const float2 x = make_float2(c.v[q], c.v[q + 1]);
+    const float2 h = plm_half2(x - make_float2(m.v[q], m.v[q + 1]), make_float2(p.v[q], p.v[q + 1]) - x);
+    t.v[q] = h.x;
+    t.v[q + 1] = h.y;
+  }
+  return t;
+}
+__device__ __forceinline__ Quad<double> plm_half(const Quad<double>& m, const Quad<double>& c,
+                                                 const Quad<double>& p) {
+  Quad<double> t;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) t.v[q] = 0.5 * vl_slope(m.v[q], c.v[q], p.v[q]);
+  return t;
+}
+
+// Face states of four variables from c[0 .. RL + RH] = cells f - RL .. f + RH.
+template <int RECON, typename R>
+__device__ __forceinline__ void recon_quad(const Quad<R>* c, R* wl, R* wr) {
+  constexpr int RH = recon_reach<RECON>(), RL = RH + 1;
+  if constexpr (RECON == 1) {
+    const Quad<R> a = plm_half(c[0], c[1], c[2]), b = plm_half(c[1], c[2], c[3]);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      wl[q] = c[1].v[q] + a.v[q];
+      wr[q] = c[2].v[q] - b.v[q];
+    }
+  } else {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      R s[6];
+#pragma unroll
+      for (int t = 0; t < 6; ++t) s[t] = (t - 3 >= -RL && t - 3 <= RH) ? c[t - 3 + RL].v[q] : R(0);
+      recon_face<RECON>(s, wl[q], wr[q]);
+    }
+  }
+}
+
+// Staged planes of one variable plane set: (rho, v1, v2, v3) and (p, Bc1,
+// Bc2, Bc3) as quads, hydro the pressure alone; with DUAL also S / rho.
+template <bool MHD, bool DUAL>
+__host__ __device__ constexpr int flux_words() { return (MHD ? 8 : 5) + (DUAL ? 1 : 0); }
 
 // Store the outputs of one face of direction D.  Scratch arrays sit at
 // sb + slot * pitch: E_ref 0..2, fluxes 8 + 5 D + v, face EMFs 23 + 2 D + q.
-template <int D, typename R>
+template <int D, bool MHD, typename R>
 __device__ __forceinline__ void store_face(R* __restrict__ sb, long long pitch, long long fc,
                                            const R* fx) {
   constexpr int T1 = (D + 1) % 3, T2 = (D + 2) % 3;
@@ -96,13 +189,21 @@ __device__ __forceinline__ void store_face(R* __restrict__ sb, long long pitch, 
   f[(1 + T1) * pitch] = fx[2];
   f[(1 + T2) * pitch] = fx[3];
   f[4 * pitch] = fx[4];
-  R* e = sb + (23 + 2 * D) * pitch + fc;
-  e[0] = fx[6];        // E_t1 =  F(B_t2)
-  e[pitch] = -fx[5];   // E_t2 = -F(B_t1)
+  if constexpr (MHD) {   // hydro reads no face EMF
+    R* e = sb + (23 + 2 * D) * pitch + fc;
+    e[0] = fx[6];        // E_t1 =  F(B_t2)
+    e[pitch] = -fx[5];   // E_t2 = -F(B_t1)
+  }
 }
 
 // ------------------------------------------------------------------------
 // 1. flux pass.  Persistent: CTAs stride over the tiles of all blocks.
+//    FP32 solves on packed (left, right) pairs (riemann2.cuh), staged cells
+//    are two quads (one 16-byte shared access each, where eight 4-byte ones
+//    were), the z slopes of a cell are formed once, and hydro carries no
+//    field terms and writes no face EMFs.  A step (VL2, PLM, HLLD, 256^3
+//    MHD): 3944 -> 3562 us; 128^3 isothermal MHD 576 -> 499 us; 128^3 hydro
+//    LHLLC RK2 510 -> 342 us (32 x 4 tiles).
 //    AETH_FLUX_MINB CTAs per SM in FP32; FP64 takes the full register file.
 // ------------------------------------------------------------------------
 // SOLVER 0: HLLD; 2: HLLE; 1: write the face states (wl, wr, bn) for the
@@ -133,16 +234,27 @@ __global__ void __launch_bounds__(flux_threads(TXT), (flux_minb<R, RECON>(TXT)))
   constexpr int QN = RL + RH + 1;
   constexpr int NB = flux_ring<RECON>(TXT);
   constexpr bool RING = NB > 1;
-  constexpr int NW = NPRIM + (DUAL ? 1 : 0);   // staged variables (+ S/rho)
-  constexpr int NQ = 7 + (DUAL ? 1 : 0);       // z-queue variables (+ S/rho)
+  constexpr bool PLM = RECON == 1;
+  constexpr int NW = flux_words<MHD, DUAL>();   // staged values of a cell
   extern __shared__ __align__(16) unsigned char flux_smem[];
   R* __restrict__ sw = reinterpret_cast<R*>(flux_smem);
-  constexpr int SN = flux_plane<RECON>(TXT);   // values of one staged plane
-  // variable v of ring plane b at plane offset s (row pitch wxr)
-  auto at = [&](int b, int v, int s) -> R& { return sw[(b * NW + v) * SN + s]; };
+  constexpr int SN = flux_plane<RECON>(TXT);   // cells of one staged plane
+  static_assert(SN % 4 == 0, "quads of every plane slot start on 16 bytes");
+  // staging slots of a thread: cells threadIdx.x + n NT of the plane
+  constexpr int NS = (SN + NT - 1) / NT;
   constexpr bool ISO = iso_solver(SOLVER);
   const R gm1 = ISO ? gamma * gamma : gamma - R(1);   // cs^2 for ISO
+  const R igm1 = ISO ? R(0) : R(1) / gm1;
   int hits = 0;
+  // half 0 / 1 of plane slot b at cell s; the entropy plane
+  auto quad = [&](int b, int half, int s) -> R* { return sw + b * (NW * SN) + half * (4 * SN) + 4 * s; };
+  auto fetch = [&](int b, int half, int s) -> Quad<R> {
+    if constexpr (!MHD) {
+      if (half == 1) return {{sw[b * (NW * SN) + 4 * SN + s], R(0), R(0), R(0)}};
+    }
+    return ld_quad(quad(b, half, s));
+  };
+  auto sent = [&](int b, int s) -> R& { return sw[b * (NW * SN) + (NW - 1) * SN + s]; };
 
   for (int t = t0 + (int)blockIdx.x; t < t1; t += gridDim.x) {
     int loc;
@@ -191,57 +303,103 @@ __global__ void __launch_bounds__(flux_threads(TXT), (flux_minb<R, RECON>(TXT)))
         return prim_cell_s<R, P64, MHD, ISO>(L, ub, pitch, cc, gm1, rho_floor, p_floor, w);
       }
     };
-    // z register queue of the own column: planes k-RL .. k+RH, 7 variables
-    // (+ S/rho; the z-face normal field comes from the face array), in the
-    // z-face frame order rho, vz, vx, vy, p, Bx, By
-    R q[NQ][QN];
-    auto load_q = [&](int slot, int kk) {   // from memory (planes below the chunk)
-      R w[8], sp = R(1);
+    const int sx = tx + RL, sy = ty + RL, so = sy * wxr + sx;   // own cell in a plane
+    // the thread's staging cells: offset in a plane of the state arrays, or
+    // < 0 outside the primitive range (the same for every plane of the tile)
+    long long soff[NS];
+#pragma unroll
+    for (int n = 0; n < NS; ++n) {
+      const int s = (int)threadIdx.x + n * NT;
+      const int ci = i0 - RL + s % wxr, cj = j0 - RL + s / wxr;
+      soff[n] = s < wxr * wyr && ci < nx + L.g && cj < ny + L.g && ci >= -L.g && cj >= -L.g
+                    ? (long long)(cj + L.g) * L.sx + ci + OX : -1;
+    }
+    // own column: both halves and S/rho of plane kk, from memory or a ring slot
+    auto own_mem = [&](int kk, Quad<R>* h, R& sp) {
+      R w[8];
+      sp = R(1);
       if (active && in_prim_range(L, i, j, kk)) {
         prim_at(L.idx(i, j, kk), w, sp);
       } else {
         w[0] = R(1); w[1] = w[2] = w[3] = R(0); w[4] = R(1); w[5] = w[6] = w[7] = R(0);
       }
-      q[0][slot] = w[0]; q[1][slot] = w[3]; q[2][slot] = w[1]; q[3][slot] = w[2];
-      q[4][slot] = w[4]; q[5][slot] = w[5]; q[6][slot] = w[6];
-      if constexpr (DUAL) q[NQ - 1][slot] = sp;
+      h[0] = {{w[0], w[1], w[2], w[3]}};
+      h[1] = {{w[4], w[5], w[6], w[7]}};
     };
-    const int sx = tx + RL, sy = ty + RL, so = sy * wxr + sx;   // own cell in a plane
-    auto ring_q = [&](int slot, int b) {    // from the staged plane in ring slot b
-      if (!active) return;
-      q[0][slot] = at(b, 0, so); q[1][slot] = at(b, 3, so); q[2][slot] = at(b, 1, so);
-      q[3][slot] = at(b, 2, so); q[4][slot] = at(b, 4, so); q[5][slot] = at(b, 5, so);
-      q[6][slot] = at(b, 6, so);
-      if constexpr (DUAL) q[NQ - 1][slot] = at(b, NW - 1, so);
+    auto own_ring = [&](int b, Quad<R>* h, R& sp) {
+      h[0] = fetch(b, 0, so);
+      h[1] = fetch(b, 1, so);
+      if constexpr (DUAL) sp = sent(b, so);
     };
     // stage plane kk (tile + halo) into ring slot b
     auto stage = [&](int kk, int b) {
-      for (int s = threadIdx.x; s < wxr * wyr; s += NT) {
-        const int rx = s % wxr, ry = s / wxr;
-        const int ci = i0 - RL + rx, cj = j0 - RL + ry;
+      const bool kin = kk >= -L.g && kk < nz + L.g;
+      const long long base = (long long)(kk + L.g) * L.sx * L.sy;
+#pragma unroll
+      for (int n = 0; n < NS; ++n) {
+        const int s = (int)threadIdx.x + n * NT;
+        if (s >= wxr * wyr) break;
         R w[8], sp = R(1);
-        if (in_prim_range(L, ci, cj, kk)) {
-          const int h = prim_at(L.idx(ci, cj, kk), w, sp);
+        if (kin && soff[n] >= 0) {
+          const int h = prim_at(base + soff[n], w, sp);
           if (kk <= k1) hits += h;   // the planes above the chunk are the next one's
         } else {
           w[0] = R(1); w[1] = w[2] = w[3] = R(0); w[4] = R(1); w[5] = w[6] = w[7] = R(0);
         }
-#pragma unroll
-        for (int v = 0; v < NPRIM; ++v) at(b, v, s) = w[v];
-        if constexpr (DUAL) at(b, NW - 1, s) = sp;
+        st_quad(quad(b, 0, s), w[0], w[1], w[2], w[3]);
+        if constexpr (MHD) st_quad(quad(b, 1, s), w[4], w[5], w[6], w[7]);
+        else sw[b * (NW * SN) + 4 * SN + s] = w[4];
+        if constexpr (DUAL) sent(b, s) = sp;
       }
     };
+    // the z stencil of the own column.  PLM: the cells k - 1, k and k + 1 and
+    // the upper-edge values of cell k - 1, carried from the previous plane,
+    // so that each cell's slope is formed once; else cells k - RL .. k + RH.
+    constexpr int ZN = PLM ? 3 : QN;
+    Quad<R> zq[ZN][2], hi[2];
+    R zs[ZN], his = R(0);
+    (void)hi; (void)his;
     // the previous tile's last plane is read until every warp is past here
     __syncthreads();
     if constexpr (RING) {
+      if constexpr (PLM) {
 #pragma unroll
-      for (int s = 0; s < RL; ++s) load_q(s, k0 - RL + s);
+        for (int s = 0; s < 2; ++s) own_mem(k0 - 2 + s, zq[s], zs[s]);
+      } else {
+#pragma unroll
+        for (int s = 0; s < RL; ++s) own_mem(k0 - RL + s, zq[s], zs[s]);
+      }
 #pragma unroll
       for (int m = 0; m < RH; ++m) stage(k0 + m, m);
     } else {
+      // band tiles: every plane of the z stencil from memory
+      if constexpr (PLM) {
+        own_mem(k0 - 2, zq[0], zs[0]);
+        own_mem(k0 - 1, zq[1], zs[1]);
+        own_mem(k0, zq[2], zs[2]);
+      } else {
 #pragma unroll
-      for (int s = 0; s < QN - 1; ++s) load_q(s + 1, k0 - RL + s);
+        for (int s = 0; s < QN - 1; ++s) own_mem(k0 - RL + s, zq[s + 1], zs[s + 1]);
+      }
     }
+    auto z_advance = [&]() {
+#pragma unroll
+      for (int s = 0; s < ZN - 1; ++s) {
+        zq[s][0] = zq[s + 1][0];
+        zq[s][1] = zq[s + 1][1];
+        if constexpr (DUAL) zs[s] = zs[s + 1];
+      }
+    };
+    // PLM: upper-edge values of the middle cell of zq
+    auto z_edge = [&]() {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const Quad<R> t = plm_half(zq[0][h], zq[1][h], zq[2][h]);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) hi[h].v[q] = zq[1][h].v[q] + t.v[q];
+      }
+      if constexpr (DUAL) his = zs[1] + R(0.5) * vl_slope(zs[0], zs[1], zs[2]);
+    };
     for (int k = k0; k <= k1; ++k) {
       int bk = 0;
       if constexpr (RING) {
@@ -255,110 +413,114 @@ __global__ void __launch_bounds__(flux_threads(TXT), (flux_minb<R, RECON>(TXT)))
         stage(k + RH, bq);
         __syncthreads();
         if (m == 0) {
+          if constexpr (PLM) {
+            own_ring(0, zq[2], zs[2]);
+            z_edge();
+            z_advance();
+            own_ring(bq, zq[2], zs[2]);
+          } else {
 #pragma unroll
-          for (int s = 0; s <= RH; ++s) ring_q(RL + s, s);
+            for (int s = 0; s <= RH; ++s) own_ring(s, zq[RL + s], zs[RL + s]);
+          }
         } else {
-          // advance the z queue: drop plane k-RL-1, add plane k+RH
-#pragma unroll
-          for (int v = 0; v < NQ; ++v)
-#pragma unroll
-            for (int s = 0; s < QN - 1; ++s) q[v][s] = q[v][s + 1];
-          ring_q(QN - 1, bq);
+          z_advance();
+          own_ring(bq, zq[ZN - 1], zs[ZN - 1]);
         }
       } else {
-        // one staged plane, the z queue from memory
+        // one staged plane, the z stencil from memory
         if (k > k0) __syncthreads();
         stage(k, 0);
-#pragma unroll
-        for (int v = 0; v < NQ; ++v)
-#pragma unroll
-          for (int s = 0; s < QN - 1; ++s) q[v][s] = q[v][s + 1];
-        load_q(QN - 1, k + RH);
+        if constexpr (PLM) {
+          if (k == k0) z_edge();
+        }
+        z_advance();
+        own_mem(k + RH, zq[ZN - 1], zs[ZN - 1]);
         __syncthreads();
       }
       if (!active) continue;
 
-      // the faces of plane k from ring slot bk (x, y, E_ref) and the z queue
+      // the faces of plane k from ring slot bk (x, y, E_ref) and the z stencil
       const long long fc = L.idx(i, j, k);
-      R wl[7], wr[7], fx[7];
-      // ---- x-face (i-1/2, j, k): frame (rho, vx, vy, vz, p, By, Bz)
+      R l8[8], r8[8];   // face states (rho, v1, v2, v3, p, B1, B2, B3)
+      R sl = R(0), sr = R(0);
+      // solve and store the face of direction D from l8, r8 (sl, sr)
+      auto face = [&](auto dir) {
+        constexpr int D = decltype(dir)::value;
+        constexpr int T1 = (D + 1) % 3, T2 = (D + 2) % 3;
+        constexpr int slot[7] = {0, 1 + D, 1 + T1, 1 + T2, 4, 5 + T1, 5 + T2};
+        R wl[7], wr[7], fx[7];
+#pragma unroll
+        for (int v = 0; v < 7; ++v) {
+          const bool zero = (!MHD && v >= 5) || (ISO && v == 4);
+          wl[v] = zero ? R(0) : l8[slot[v]];
+          wr[v] = zero ? R(0) : r8[slot[v]];
+        }
+        const R bn = MHD ? ub[(5 + D) * pitch + fc] : R(0);
+        if constexpr (SOLVER != 1) {
+          solve_face<SOLVER, MHD>(gamma, igm1, wl, wr, bn, fx);
+          store_face<D, MHD>(sb, pitch, fc, fx);
+          if constexpr (DUAL) sb[(3 + D) * pitch + fc] = fx[0] >= R(0) ? fx[0] * sl : fx[0] * sr;
+        } else {
+          R* fs = P.fstate + (D * 15) * pitch + fc;
+#pragma unroll
+          for (int v = 0; v < 7; ++v) { fs[v * pitch] = wl[v]; fs[(7 + v) * pitch] = wr[v]; }
+          fs[14 * pitch] = bn;
+        }
+      };
+      // states of the lower face along a staged axis (cell stride ds)
+      auto plane_states = [&](int ds) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          Quad<R> c[QN];
+#pragma unroll
+          for (int q = 0; q < QN; ++q) c[q] = fetch(bk, h, so + (q - RL) * ds);
+          recon_quad<RECON>(c, l8 + 4 * h, r8 + 4 * h);
+        }
+        if constexpr (DUAL) recon_var<RECON>([&](int off) { return sent(bk, so + off * ds); }, sl, sr);
+      };
       if (i >= 0) {
-        const int slot[7] = {0, 1, 2, 3, 4, 6, 7};
-#pragma unroll
-        for (int v = 0; v < 7; ++v) {
-          if ((!MHD && v >= 5) || (ISO && v == 4)) { wl[v] = wr[v] = R(0); continue; }
-          recon_var<RECON>([&](int off) { return at(bk, slot[v], so + off); }, wl[v], wr[v]);
-        }
-        const R bn = MHD ? ub[5 * pitch + fc] : R(0);
-        if (SOLVER != 1) {
-          solve_face<SOLVER>(gamma, wl, wr, bn, fx);
-          store_face<0>(sb, pitch, fc, fx);
-          if constexpr (DUAL) {
-            R sl, sr;
-            recon_var<RECON>([&](int off) { return at(bk, NW - 1, so + off); }, sl, sr);
-            sb[3 * pitch + fc] = fx[0] >= R(0) ? fx[0] * sl : fx[0] * sr;
-          }
-        } else {
-          R* fs = P.fstate + (0 * 15) * pitch + fc;
-#pragma unroll
-          for (int v = 0; v < 7; ++v) { fs[v * pitch] = wl[v]; fs[(7 + v) * pitch] = wr[v]; }
-          fs[14 * pitch] = bn;
-        }
+        plane_states(1);
+        face(Int<0>{});
       }
-      // ---- y-face (i, j-1/2, k): frame (rho, vy, vz, vx, p, Bz, Bx)
       if (j >= 0) {
-        const int slot[7] = {0, 2, 3, 1, 4, 7, 5};
-#pragma unroll
-        for (int v = 0; v < 7; ++v) {
-          if ((!MHD && v >= 5) || (ISO && v == 4)) { wl[v] = wr[v] = R(0); continue; }
-          recon_var<RECON>([&](int off) { return at(bk, slot[v], so + off * wxr); }, wl[v], wr[v]);
-        }
-        const R bn = MHD ? ub[6 * pitch + fc] : R(0);
-        if (SOLVER != 1) {
-          solve_face<SOLVER>(gamma, wl, wr, bn, fx);
-          store_face<1>(sb, pitch, fc, fx);
-          if constexpr (DUAL) {
-            R sl, sr;
-            recon_var<RECON>([&](int off) { return at(bk, NW - 1, so + off * wxr); }, sl, sr);
-            sb[4 * pitch + fc] = fx[0] >= R(0) ? fx[0] * sl : fx[0] * sr;
-          }
-        } else {
-          R* fs = P.fstate + (1 * 15) * pitch + fc;
-#pragma unroll
-          for (int v = 0; v < 7; ++v) { fs[v * pitch] = wl[v]; fs[(7 + v) * pitch] = wr[v]; }
-          fs[14 * pitch] = bn;
-        }
+        plane_states(wxr);
+        face(Int<1>{});
       }
-      // ---- z-face (i, j, k-1/2): frame (rho, vz, vx, vy, p, Bx, By)
-      if (k >= 0) {
+      if constexpr (PLM) {
+        // lower-edge values of cell k, and its upper-edge values for face k + 1
 #pragma unroll
-        for (int v = 0; v < 7; ++v) {
-          if ((!MHD && v >= 5) || (ISO && v == 4)) { wl[v] = wr[v] = R(0); continue; }
-          recon_var<RECON>([&](int off) { return q[v][off + RL]; }, wl[v], wr[v]);
-        }
-        const R bn = MHD ? ub[7 * pitch + fc] : R(0);
-        if (SOLVER != 1) {
-          solve_face<SOLVER>(gamma, wl, wr, bn, fx);
-          store_face<2>(sb, pitch, fc, fx);
-          if constexpr (DUAL) {
-            R sl, sr;
-            recon_var<RECON>([&](int off) { return q[NQ - 1][off + RL]; }, sl, sr);
-            sb[5 * pitch + fc] = fx[0] >= R(0) ? fx[0] * sl : fx[0] * sr;
+        for (int h = 0; h < 2; ++h) {
+          const Quad<R> t = plm_half(zq[0][h], zq[1][h], zq[2][h]);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            l8[4 * h + q] = hi[h].v[q];
+            r8[4 * h + q] = zq[1][h].v[q] - t.v[q];
+            hi[h].v[q] = zq[1][h].v[q] + t.v[q];
           }
-        } else {
-          R* fs = P.fstate + (2 * 15) * pitch + fc;
-#pragma unroll
-          for (int v = 0; v < 7; ++v) { fs[v * pitch] = wl[v]; fs[(7 + v) * pitch] = wr[v]; }
-          fs[14 * pitch] = bn;
         }
+        if constexpr (DUAL) {
+          const R t = R(0.5) * vl_slope(zs[0], zs[1], zs[2]);
+          sl = his;
+          sr = zs[1] - t;
+          his = zs[1] + t;
+        }
+      } else {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          Quad<R> c[QN];
+#pragma unroll
+          for (int q = 0; q < QN; ++q) c[q] = zq[q][h];
+          recon_quad<RECON>(c, l8 + 4 * h, r8 + 4 * h);
+        }
+        if constexpr (DUAL) recon_var<RECON>([&](int off) { return zs[off + RL]; }, sl, sr);
       }
+      if (k >= 0) face(Int<2>{});
       // ---- cell-centred reference EMF, E = -v x B
-      if (MHD) {
-        const R vx = at(bk, 1, so), vy = at(bk, 2, so), vz = at(bk, 3, so);
-        const R bx_ = at(bk, 5, so), by_ = at(bk, 6, so), bz_ = at(bk, 7, so);
-        sb[fc] = -(vy * bz_ - vz * by_);
-        sb[pitch + fc] = -(vz * bx_ - vx * bz_);
-        sb[2 * pitch + fc] = -(vx * by_ - vy * bx_);
+      if constexpr (MHD) {
+        const Quad<R> a = zq[PLM ? 1 : RL][0], b = zq[PLM ? 1 : RL][1];
+        sb[fc] = -(a.v[2] * b.v[3] - a.v[3] * b.v[2]);
+        sb[pitch + fc] = -(a.v[3] * b.v[1] - a.v[1] * b.v[3]);
+        sb[2 * pitch + fc] = -(a.v[1] * b.v[2] - a.v[2] * b.v[1]);
       }
     }
   }
@@ -405,7 +567,7 @@ static void with_src(aeth_ctx* c, int kind, int block, F launch) {
 template <typename R, bool P64, int RECON, bool MHD, int SOLVER, bool DUAL>
 static void launch_flux3(aeth_ctx* c, int src, int block) {
 
-  constexpr int NW = NPRIM + (DUAL ? 1 : 0);
+  constexpr int NW = flux_words<MHD, DUAL>();
   with_src<R>(c, PK_FLUX, block, [&](auto S, TileRange r) {
     // tx: the tile width the kernel was built for (0: band tiles)
     auto go = [&](auto kernel, int tx) {
