@@ -1,5 +1,6 @@
 // Ghost fill (Sec. 2.3), host<->device state conversion, the CFL reduction
 // of Eq. 11 and the FP64 history diagnostics, for every working precision.
+#include <algorithm>
 #include <cmath>
 
 #include "runtime.hpp"
@@ -157,20 +158,44 @@ aeth_status build_geometry(aeth_ctx* c) {
   return c->elem == 8 ? build_geometry_T<double>(c) : build_geometry_T<float>(c);
 }
 
-// Device block table and the tile prefix sums of every pass kind.
-// Default z extent of a flux tile: the largest of {64, 32, 16, 8, 4} that
-// still gives every SM at least four tiles (small grids need short
-// chunks to fill the GPU; long chunks amortise the z-halo warm-up).
+// Default z extent of a flux tile.  A tile of kc planes costs kc + w plane
+// units (w: the stencil planes below the chunk and the first copies); a chip
+// that runs `slots` tiles at a time takes about the mean load of a slot plus
+// half a tile for the end of the last wave, and at least one tile.  Measured
+// with 32-wide tiles, us per step: 256^3 FP32 3075 (kc 8), 3063 (17), 3079
+// (30), 3150 (64); 128^3 isothermal 458 (8), 459 (17), 475 (32); 64^3 113 (1),
+// 109 (2 to 6); 32^3 68 (1), 72 (4), 78 (6); FP64 96^3 6960 (4), 7283 (7), 7743
+// (16).  The longest chunk with four tiles an SM, the rule before, took 64, 32
+// and 16 of these.
 static int default_kchunk(const aeth_ctx* c) {
-  const int want = 4 * c->num_sms;
-  for (int kc : {64, 32, 16, 8, 4}) {
-    long long tiles = 0;
-    for (const auto& B : c->blocks) tiles += tiles_of(B.L, PK_FLUX, kc, c->flux_tx);
-    if (tiles >= want) return kc;
+  int nzmax = 1;
+  for (const auto& B : c->blocks) nzmax = std::max(nzmax, B.L.n[2]);
+  // FP64: the FP64 pipe of an SM, not a slot, is the unit that runs out, so a
+  // whole tile ends late; staging costs next to nothing there
+  const bool f64 = c->elem == 8;
+  const double slots = (double)c->num_sms * (f64 ? 2 : (c->flux_tx ? 5 : 2));
+  const double w = f64 ? 0.3 : 1.0, tail = f64 ? 1.0 : 0.5;
+  int best = 1;
+  double best_cost = 1e300;
+  // the even divisions of the tallest block
+  for (int parts = 1; parts <= nzmax + 2; ++parts) {
+    const int kc = ceil_div(nzmax + 2, parts);
+    if (kc > 64 || ceil_div(nzmax + 2, kc) != parts) continue;
+    double planes = 0;
+    for (const auto& B : c->blocks) {
+      const double chunks = ceil_div(B.L.n[2] + 2, kc);
+      planes += tiles_of(B.L, PK_FLUX, kc, c->flux_tx) / chunks * (B.L.n[2] + 2 + w * chunks);
+    }
+    const double cost = std::max(kc + w, planes / slots + tail * (kc + w));
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = kc;
+    }
   }
-  return 4;
+  return best;
 }
 
+// Device block table and the tile prefix sums of every pass kind.
 template <typename R>
 static aeth_status build_tables_T(aeth_ctx* c) {
   const int nb = (int)c->blocks.size();

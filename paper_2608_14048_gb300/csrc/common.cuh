@@ -72,6 +72,19 @@ template <typename R> __device__ __forceinline__ R rsqrt_(R x);
 template <> __device__ __forceinline__ double rsqrt_(double x) { return 1.0 / sqrt(x); }
 template <> __device__ __forceinline__ float rsqrt_(float x) { return 1.0f / sqrtf(x); }
 
+// Reciprocal and quotient.  FP32: the hardware reciprocal (1 ulp) and one
+// multiplication, which is also what the division operator returns under
+// -prec-div=false (bit for bit on 3e9 operand pairs of exponents -60 .. 60)
+// after scaling its operands; FP64: the division.
+__device__ __forceinline__ double recip(double x) { return 1.0 / x; }
+__device__ __forceinline__ float recip(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ double quot(double a, double b) { return a / b; }
+__device__ __forceinline__ float quot(float a, float b) { return __fmul_rn(a, recip(b)); }
+
 // ------------------------------------------------------------------------
 // Reconstruction (Sec. 2.4)
 // ------------------------------------------------------------------------
@@ -166,6 +179,20 @@ __device__ __forceinline__ R fast_speed(R gamma, R rho, R p, R bn, R bt1, R bt2)
   // one reciprocal of rho for the three quotients
   const R ir = R(1) / rho;
   const R a2 = gamma * p * ir;
+  const R b2 = (bn * bn + bt1 * bt1 + bt2 * bt2) * ir;
+  const R s = a2 + b2;
+  const R disc = fmax(s * s - R(4) * a2 * bn * bn * ir, R(0));
+  return sqrt(R(0.5) * (s + sqrt(disc)));
+}
+
+// The fast speed of the HLLE solvers: the same bits with the reciprocal above;
+// MHD = false, without field: the expression at zero field (every dropped
+// term is a product with zero).
+template <bool MHD, typename R>
+__device__ __forceinline__ R fast_speed_of(R gamma, R rho, R p, R bn, R bt1, R bt2) {
+  const R ir = recip(rho);
+  const R a2 = gamma * p * ir;
+  if constexpr (!MHD) return sqrt(R(0.5) * (a2 + sqrt(fmax(a2 * a2, R(0)))));
   const R b2 = (bn * bn + bt1 * bt1 + bt2 * bt2) * ir;
   const R s = a2 + b2;
   const R disc = fmax(s * s - R(4) * a2 * bn * bn * ir, R(0));
@@ -335,11 +362,18 @@ __device__ __forceinline__ int hlld(R gamma, const R* wl, const R* wr, R bn, R* 
 // HLLD solver, S_L = min(vn) - max(c_f), S_R = max(vn) + max(c_f), with
 // b- = min(S_L, 0), b+ = max(S_R, 0) (a supersonic face takes the upwind
 // flux without a branch).  Same frames as hlld; returns 0.
-template <typename R>
+template <bool MHD = true, typename R>
 __device__ __forceinline__ int hlle(R gamma, const R* wl, const R* wr, R bn, R* f) {
-  const R igm1 = R(1) / (gamma - R(1));
+  const R igm1 = recip(gamma - R(1));
   auto side = [&](const R* w, R* u, R* fx) {
     const R rho = w[0], vn = w[1], v1 = w[2], v2 = w[3], p = w[4], b1 = w[5], b2 = w[6];
+    if constexpr (!MHD) {   // the same without field, bit for bit
+      const R e = p * igm1 + R(0.5) * rho * (vn * vn + v1 * v1 + v2 * v2);
+      u[0] = rho; u[1] = rho * vn; u[2] = rho * v1; u[3] = rho * v2; u[4] = e;
+      fx[0] = rho * vn; fx[1] = rho * vn * vn + p; fx[2] = rho * vn * v1; fx[3] = rho * vn * v2;
+      fx[4] = (e + p) * vn;
+      return;
+    }
     const R bb = bn * bn + b1 * b1 + b2 * b2;
     const R pt = p + R(0.5) * bb;
     const R e = p * igm1 + R(0.5) * rho * (vn * vn + v1 * v1 + v2 * v2) + R(0.5) * bb;
@@ -352,13 +386,14 @@ __device__ __forceinline__ int hlle(R gamma, const R* wl, const R* wr, R bn, R* 
   R ul[7], ur[7], fl[7], fr[7];
   side(wl, ul, fl);
   side(wr, ur, fr);
-  const R cm = fmax(fast_speed(gamma, wl[0], wl[4], bn, wl[5], wl[6]),
-                    fast_speed(gamma, wr[0], wr[4], bn, wr[5], wr[6]));
+  const R cm = fmax(fast_speed_of<MHD>(gamma, wl[0], wl[4], bn, wl[5], wl[6]),
+                    fast_speed_of<MHD>(gamma, wr[0], wr[4], bn, wr[5], wr[6]));
   const R bm = fmin(fmin(wl[1], wr[1]) - cm, R(0));
   const R bp = fmax(fmax(wl[1], wr[1]) + cm, R(0));
-  const R inv = R(1) / (bp - bm);
+  const R inv = recip(bp - bm);
+  if constexpr (!MHD) f[5] = f[6] = R(0);
 #pragma unroll
-  for (int q = 0; q < 7; ++q) f[q] = (bp * fl[q] - bm * fr[q] + bp * bm * (ur[q] - ul[q])) * inv;
+  for (int q = 0; q < (MHD ? 7 : 5); ++q) f[q] = (bp * fl[q] - bm * fr[q] + bp * bm * (ur[q] - ul[q])) * inv;
   return 0;
 }
 
@@ -367,35 +402,42 @@ __device__ __forceinline__ int hlle(R gamma, const R* wl, const R* wr, R bn, R* 
 // (energy entries zero) and the outer speeds (the fast speed with gamma = 1
 // and p = cs^2 rho).
 // ------------------------------------------------------------------------
-template <typename R>
+template <bool MHD = true, typename R>
 __device__ __forceinline__ void side_iso(R a2, const R* w, R bn, R* u, R* f) {
   const R rho = w[0], vn = w[1], v1 = w[2], v2 = w[3], b1 = w[5], b2 = w[6];
+  if constexpr (!MHD) {   // the same without field, bit for bit
+    u[0] = rho; u[1] = rho * vn; u[2] = rho * v1; u[3] = rho * v2;
+    f[0] = rho * vn; f[1] = rho * vn * vn + a2 * rho; f[2] = rho * vn * v1; f[3] = rho * vn * v2;
+    u[4] = u[5] = u[6] = f[4] = f[5] = f[6] = R(0);
+    return;
+  }
   const R pt = a2 * rho + R(0.5) * (bn * bn + b1 * b1 + b2 * b2);
   u[0] = rho; u[1] = rho * vn; u[2] = rho * v1; u[3] = rho * v2; u[4] = R(0); u[5] = b1; u[6] = b2;
   f[0] = rho * vn; f[1] = rho * vn * vn + pt - bn * bn; f[2] = rho * vn * v1 - bn * b1;
   f[3] = rho * vn * v2 - bn * b2; f[4] = R(0); f[5] = b1 * vn - bn * v1; f[6] = b2 * vn - bn * v2;
 }
 
-template <typename R>
+template <bool MHD = true, typename R>
 __device__ __forceinline__ void iso_speeds(R a2, const R* wl, const R* wr, R bn, R& sl, R& sr) {
-  const R cm = fmax(fast_speed(R(1), wl[0], a2 * wl[0], bn, wl[5], wl[6]),
-                    fast_speed(R(1), wr[0], a2 * wr[0], bn, wr[5], wr[6]));
+  const R cm = fmax(fast_speed_of<MHD>(R(1), wl[0], a2 * wl[0], bn, wl[5], wl[6]),
+                    fast_speed_of<MHD>(R(1), wr[0], a2 * wr[0], bn, wr[5], wr[6]));
   sl = fmin(wl[1], wr[1]) - cm;
   sr = fmax(wl[1], wr[1]) + cm;
 }
 
 // Isothermal HLLE: HLL average between the outer speeds (branch-free form).
-template <typename R>
+template <bool MHD = true, typename R>
 __device__ __forceinline__ int hlle_iso(R cs, const R* wl, const R* wr, R bn, R* f) {
   const R a2 = cs * cs;
   R ul[7], ur[7], fl[7], fr[7], sl, sr;
-  side_iso(a2, wl, bn, ul, fl);
-  side_iso(a2, wr, bn, ur, fr);
-  iso_speeds(a2, wl, wr, bn, sl, sr);
+  side_iso<MHD>(a2, wl, bn, ul, fl);
+  side_iso<MHD>(a2, wr, bn, ur, fr);
+  iso_speeds<MHD>(a2, wl, wr, bn, sl, sr);
   const R bm = fmin(sl, R(0)), bp = fmax(sr, R(0));
-  const R inv = R(1) / (bp - bm);
+  const R inv = recip(bp - bm);
+  if constexpr (!MHD) f[4] = f[5] = f[6] = R(0);
 #pragma unroll
-  for (int q = 0; q < 7; ++q) f[q] = (bp * fl[q] - bm * fr[q] + bp * bm * (ur[q] - ul[q])) * inv;
+  for (int q = 0; q < (MHD ? 7 : 4); ++q) f[q] = (bp * fl[q] - bm * fr[q] + bp * bm * (ur[q] - ul[q])) * inv;
   return 0;
 }
 

@@ -1,314 +1,261 @@
-// FP32 face solvers and PLM reconstruction of the flux pass on packed pairs.
+// FP32 face solvers of the flux pass on packed (left, right) pairs.
 //
-// The flux pass is bound by instruction issue (no pipe near its peak, other
-// warps ready when one waits), and sm_103a executes two FP32 additions,
-// multiplications or FMAs of a lane in one packed instruction (f32x2).  A
-// Riemann solver does the same arithmetic for the left and the right state,
-// so the pair (left, right) is the packed operand from the reconstruction to
-// the choice of the region; only that choice and the double-star states are
-// scalar.  Reciprocals are the hardware approximation (1 ulp) and one
-// multiplication, where the division operator scales its operands first.
-//
-// Measured with the scalar solvers (division and square-root operators, one
-// 4-byte shared load a value) before and these after, us per launch of the
-// PLM corrector: see k_flux3.
+// The flux pass is bound by instruction issue, and a Riemann solver does the
+// same arithmetic for the left and the right state: the pair is the packed
+// operand (pair.cuh) from the reconstruction to the choice of the region; only
+// that choice and the double-star states are scalar.
 //
 // The formulas are those of common.cuh's scalar solvers, which FP64, the
-// unfused path and the learned flux's fallback use; MHD = false drops every
-// field term, which the scalar solvers carry as zeros.
+// unfused path and the learned flux's fallback use.  Every rounding is written
+// out (which product of a sum enters a fused multiply-add, and which is
+// rounded by itself), so that a face's flux does not depend on what the
+// compiler fuses in one instantiation and not in the next: shocks and limiters
+// amplify a last-bit difference, and results stay comparable bit for bit
+// across tile shapes, block layouts and versions of the kernel around them.
+// MHD = false drops every field term (a product with zero) with the same bits.
 #pragma once
-#include "common.cuh"
+#include "pair.cuh"
 
 namespace aeth {
 
-__device__ __forceinline__ float2 splat(float a) { return make_float2(a, a); }
-__device__ __forceinline__ float2 operator+(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 operator*(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 operator-(float2 a, float2 b) {
-  float2 r;
-  asm("{\n\t.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\t"
-      "sub.rn.ftz.f32x2 z, x, y;\n\tmov.b64 {%0, %1}, z;\n\t}"
-      : "=f"(r.x), "=f"(r.y)
-      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-  return r;
+__device__ __forceinline__ float rmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float radd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float rsub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float rfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+// A product that a sum takes in rounded: as two scalar multiplications (a packed
+// one is fused into the packed sum that follows, whatever its rounding says).
+__device__ __forceinline__ float2 mul_apart(float2 a, float2 b) {
+  return make_float2(rmul(a.x, b.x), rmul(a.y, b.y));
 }
+__device__ __forceinline__ float pick(bool left, float2 a) { return left ? a.x : a.y; }
 
-__device__ __forceinline__ float rcp_(float x) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-__device__ __forceinline__ float sqrt_(float x) {
-  float r;
-  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-__device__ __forceinline__ float2 rcp2(float2 a) { return make_float2(rcp_(a.x), rcp_(a.y)); }
-__device__ __forceinline__ float2 sqrt2(float2 a) { return make_float2(sqrt_(a.x), sqrt_(a.y)); }
-
-// Half the van Leer slope of two variables at once: dm dp / (dm + dp) where
-// the differences have one sign, else 0.
-__device__ __forceinline__ float2 plm_half2(float2 dm, float2 dp) {
-  const float2 q = dm * dp, r = rcp2(dm + dp);
-  const float2 t = q * r;
-  return make_float2(q.x > 0.0f ? t.x : 0.0f, q.y > 0.0f ? t.y : 0.0f);
-}
-
-// One side pair: conserved vector and physical flux of (left, right), total
-// pressure and fast speed.  W = (rho, vn, vt1, vt2, p, Bt1, Bt2).
+// Conserved vector, physical flux, total pressure and fast speed of the pair;
+// W = (rho, vn, vt1, vt2, p, Bt1, Bt2).  g: gamma (ISO: cs^2); igm1 =
+// 1 / (gamma - 1) (the pressure is divided by gamma - 1 as one product).
 template <bool MHD, bool ISO>
 struct SidePair {
-  float2 u2, u3, e;                     // rho vt1, rho vt2, total energy
-  float2 f0, f1, f2, f3, f4, f5, f6;    // physical flux (f0 = rho vn)
+  float2 nrho, nun;                    // -rho, -vn
+  float2 e, vv;                        // total energy, |v|^2
+  float2 f0, f1, f2, f3, f4, f5, f6;   // physical flux (f0 = rho vn)
+  float2 f1t;                          // f1 before the subtraction of bn^2
   float2 pt, vb, cf;
 
-  // g: gamma (ISO: the sound speed squared); igm1 = 1 / (gamma - 1)
   __device__ __forceinline__ SidePair(float g, float igm1, const float2* W, float bn, float bn2) {
     const float2 rho = W[0], un = W[1], v1 = W[2], v2 = W[3], b1 = W[5], b2 = W[6];
-    const float2 ir = rcp2(rho), B = splat(bn), nB = splat(-bn);
+    nrho = make_float2(-rho.x, -rho.y);
+    nun = make_float2(-un.x, -un.y);
+    const float2 ir = make_float2(recip(rho.x), recip(rho.y));
     const float2 p = ISO ? splat(g) * rho : W[4];
+    const float2 a2 = (ISO ? p : splat(g) * p) * ir;
     f0 = rho * un;
-    u2 = rho * v1;
-    u3 = rho * v2;
     if constexpr (MHD) {
+      const float2 B = splat(bn), nB = splat(-bn);
       const float2 bb = fma2(b2, b2, fma2(b1, b1, splat(bn2)));
-      pt = fma2(bb, splat(0.5f), p);
-      f1 = fma2(f0, un, pt - splat(bn2));
-      f2 = fma2(u2, un, nB * b1);
-      f3 = fma2(u3, un, nB * b2);
+      if constexpr (ISO) pt = fma2(splat(g), rho, splat(0.5f) * bb);
+      else pt = fma2(splat(0.5f), bb, p);
+      f1t = fma2(f0, un, pt);
+      f1 = f1t - splat(bn2);
+      f2 = fma2(f0, v1, nB * b1);
+      f3 = fma2(f0, v2, nB * b2);
       f5 = fma2(b1, un, nB * v1);
       f6 = fma2(b2, un, nB * v2);
-      const float2 a2 = ISO ? splat(g) : p * (splat(g) * ir);
       const float2 s = fma2(bb, ir, a2);
-      const float2 disc = fma2(s, s, (a2 * ir) * splat(-4.0f * bn2));
-      const float2 root = sqrt2(make_float2(fmaxf(disc.x, 0.0f), fmaxf(disc.y, 0.0f)));
-      cf = sqrt2((s + root) * splat(0.5f));
+      const float2 disc = fma2(s, s, (((splat(-4.0f) * a2) * B) * B) * ir);
+      cf = speed(s, disc);
       if constexpr (!ISO) {
-        vb = fma2(v2, b2, fma2(v1, b1, un * B));
-        const float2 k = fma2(u3, v2, fma2(u2, v1, f0 * un));
-        e = fma2(p, splat(igm1), (k + bb) * splat(0.5f));
+        vb = fma2(v2, b2, fma2(un, B, v1 * b1));
+        vv = fma2(v2, v2, fma2(un, un, v1 * v1));
+        e = fma2(splat(0.5f), bb, fma2(splat(0.5f) * rho, vv, p * splat(igm1)));
         f4 = fma2(e + pt, un, nB * vb);
       }
     } else {
       pt = p;
-      f1 = fma2(f0, un, pt);
-      f2 = u2 * un;
-      f3 = u3 * un;
-      if constexpr (ISO) {
-        cf = splat(sqrt_(g));
-      } else {
-        cf = sqrt2(p * (splat(g) * ir));
-        const float2 k = fma2(u3, v2, fma2(u2, v1, f0 * un));
-        e = fma2(p, splat(igm1), k * splat(0.5f));
+      f1 = f1t = fma2(f0, un, pt);
+      f2 = f0 * v1;
+      f3 = f0 * v2;
+      cf = speed(a2, a2 * a2);
+      if constexpr (!ISO) {
+        vv = fma2(v2, v2, fma2(un, un, v1 * v1));
+        e = fma2(splat(0.5f) * rho, vv, p * splat(igm1));
         f4 = (e + pt) * un;
       }
     }
   }
+  static __device__ __forceinline__ float2 speed(float2 s, float2 disc) {
+    const float2 r = make_float2(sqrtf(fmaxf(disc.x, 0.0f)), sqrtf(fmaxf(disc.y, 0.0f)));
+    const float2 h = splat(0.5f) * (s + r);
+    return make_float2(sqrtf(h.x), sqrtf(h.y));
+  }
 };
 
-// HLLD (hlld_s of common.cuh; LD: LHLLD).  MHD = false: HLLC / LHLLC.
-template <bool LD, bool MHD>
+// HLLD (hlld_s of common.cuh; LD: LHLLD); MHD = false: HLLC / LHLLC.  SPLIT:
+// the right side's normal momentum flux subtracts a rounded bn^2 like the left
+// side's, instead of fusing the product.
+template <bool LD, bool MHD, bool SPLIT>
 __device__ __forceinline__ void hlld2(float gamma, float igm1, const float2* W, float bn, float* f) {
-  const float bn2 = bn * bn;
+  const float bn2 = rmul(bn, bn);
   const SidePair<MHD, false> P(gamma, igm1, W, bn, bn2);
   const float2 rho = W[0], un = W[1], v1 = W[2], v2 = W[3], b1 = W[5], b2 = W[6];
   const float cmax = fmaxf(P.cf.x, P.cf.y);
-  const float2 S = make_float2(fminf(un.x, un.y) - cmax, fmaxf(un.x, un.y) + cmax);
+  const float2 S = make_float2(rsub(fminf(un.x, un.y), cmax), radd(fmaxf(un.x, un.y), cmax));
   if constexpr (!MHD) f[5] = f[6] = 0.0f;
   if (S.x > 0.0f || S.y < 0.0f) {   // supersonic: the upwind side's flux
     const bool l = S.x > 0.0f;
-    f[0] = l ? P.f0.x : P.f0.y;
-    f[1] = l ? P.f1.x : P.f1.y;
-    f[2] = l ? P.f2.x : P.f2.y;
-    f[3] = l ? P.f3.x : P.f3.y;
-    f[4] = l ? P.f4.x : P.f4.y;
-    if constexpr (MHD) {
-      f[5] = l ? P.f5.x : P.f5.y;
-      f[6] = l ? P.f6.x : P.f6.y;
-    }
+    f[0] = pick(l, P.f0); f[1] = pick(l, P.f1); f[2] = pick(l, P.f2); f[3] = pick(l, P.f3);
+    f[4] = pick(l, P.f4);
+    if constexpr (MHD) { f[5] = pick(l, P.f5); f[6] = pick(l, P.f6); }
     return;
   }
-  const float2 su = S - un, m = rho * su;
-  const float iden = rcp_(m.y - m.x);
-  const float sm = (fmaf(m.y, un.y, -m.x * un.x) + (P.pt.x - P.pt.y)) * iden;
-  const float du = un.y - un.x, mm = m.x * m.y;
-  const float pts = fmaf(mm, du, fmaf(m.y, P.pt.x, -m.x * P.pt.y)) * iden;
-  const float2 sm2 = splat(sm), ss = S - sm2, iss = rcp2(ss);
+  const float2 su = S - un, m = su * rho;
+  const float iden = recip(rsub(m.y, m.x));
+  const float sm = rmul(radd(rsub(rfma(m.y, un.y, rmul(m.x, P.nun.x)), P.pt.y), P.pt.x), iden);
+  const float t5 = rmul(rmul(rmul(rho.x, rho.y), su.y), su.x), du = rsub(un.y, un.x);
+  const float x = rfma(m.y, P.pt.x, -rmul(m.x, P.pt.y));
+  const float pts = rmul(LD ? radd(rmul(t5, du), x) : rfma(t5, du, x), iden);
+  const float2 ss = S - splat(sm), iss = make_float2(recip(ss.x), recip(ss.y));
   const float2 rs = m * iss;
-  float ld1 = 0.0f;   // LHLLD: the change of the pressure dissipation
+  // star energy, without the field's work in hydro
+  const float2 ea = fma2(su, P.e, P.pt * P.nun), eb = splat(rmul(pts, sm)) + ea;
+  float pd = 0.0f;   // LHLLD: the change of the pressure dissipation
   if constexpr (LD) {
-    const float2 vm = sqrt2(fma2(v2, v2, fma2(v1, v1, un * un)));
-    const float phi = fminf(1.0f, fmaxf(vm.x, vm.y) * rcp_(cmax));
-    ld1 = (phi - 1.0f) * (mm * du * iden);
+    const float phi = fminf(1.0f, rmul(fmaxf(sqrtf(P.vv.x), sqrtf(P.vv.y)), recip(cmax)));
+    pd = rmul(rsub(phi, 1.0f), rmul(rmul(t5, du), iden));
   }
+  // F* = F + S (U* - U) of both sides
+  const float2 g0 = fma2(S, rs - rho, P.f0);
+  const float2 d1 = fma2(rs, splat(sm), rho * P.nun);
   if constexpr (!MHD) {
-    // one star state a side, transverse velocities unchanged
-    const float2 es = (fma2(su, P.e, splat(pts * sm)) - P.pt * un) * iss;
-    const float2 dr = rs - rho;
-    const float2 g0 = fma2(S, dr, P.f0), g1 = fma2(S, rs * sm2 - P.f0, P.f1);
-    const float2 sd = S * dr;
-    const float2 g2 = fma2(sd, v1, P.f2), g3 = fma2(sd, v2, P.f3), g4 = fma2(S, es - P.e, P.f4);
+    const float2 es = mul_apart(eb, iss);
+    const float2 g1 = fma2(S, d1, P.f1);
+    const float2 g2 = fma2(S, fma2(P.nrho, v1, rs * v1), P.f2);
+    const float2 g3 = fma2(S, fma2(P.nrho, v2, rs * v2), P.f3);
+    const float2 g4 = fma2(S, es - P.e, P.f4);
     const bool l = sm >= 0.0f;
-    f[0] = l ? g0.x : g0.y;
-    f[1] = (l ? g1.x : g1.y) + ld1;
-    f[2] = l ? g2.x : g2.y;
-    f[3] = l ? g3.x : g3.y;
-    f[4] = fmaf(ld1, sm, l ? g4.x : g4.y);
-    return;
+    f[0] = pick(l, g0);
+    f[1] = LD ? radd(pick(l, g1), pd) : pick(l, g1);
+    f[2] = pick(l, g2);
+    f[3] = pick(l, g3);
+    f[4] = LD ? rfma(pd, sm, pick(l, g4)) : pick(l, g4);
   } else {
-    const float2 dd = fma2(m, ss, splat(-bn2)), idd = rcp2(dd);
-    const float2 bni = splat(bn) * idd;
-    float2 nfv = bni * (un - sm2);                       // -(transverse velocity factor)
-    float2 fb = fma2(m, su, splat(-bn2)) * idd;
-    const float lim = Eps<float>::hlld * pts;
+    const float2 nbn2 = splat(-bn2);
+    const float2 dd = fma2(m, ss, nbn2), idd = make_float2(recip(dd.x), recip(dd.y));
+    float2 nfv = (splat(bn) * (un - splat(sm))) * idd;   // -(transverse velocity factor)
+    float2 fb = fma2(m, su, nbn2) * idd;
+    const float lim = rmul(Eps<float>::hlld, pts);
     if (fabsf(dd.x) < lim) { nfv.x = 0.0f; fb.x = 1.0f; }
     if (fabsf(dd.y) < lim) { nfv.y = 0.0f; fb.y = 1.0f; }
     const float2 v1s = fma2(b1, nfv, v1), v2s = fma2(b2, nfv, v2), b1s = b1 * fb, b2s = b2 * fb;
-    const float2 vbs = fma2(v2s, b2s, fma2(v1s, b1s, splat(sm * bn)));
-    const float2 es = fma2(splat(bn), P.vb - vbs, fma2(su, P.e, splat(pts * sm)) - P.pt * un) * iss;
+    const float smb = rmul(sm, bn);
+    const float2 vbs = fma2(v2s, b2s, fma2(v1s, b1s, splat(smb)));
+    const float2 es = fma2(splat(bn), P.vb - vbs, eb) * iss;
     const float2 q = make_float2(rsqrtf(rs.x), rsqrtf(rs.y)), sq = rs * q;
     const float abn = fabsf(bn);
-    const bool degen = 0.5f * bn2 < lim;
-    const float ssl = degen ? sm : fmaf(-abn, q.x, sm);
-    const float ssr = degen ? sm : fmaf(abn, q.y, sm);
-    // F* = F + S (U* - U) of both sides
-    const float2 rv1 = rs * v1s, rv2 = rs * v2s;
-    const float2 g0 = fma2(S, rs - rho, P.f0);
-    const float2 g1 = fma2(S, rs * sm2 - P.f0, P.f1);
-    const float2 g2 = fma2(S, rv1 - P.u2, P.f2), g3 = fma2(S, rv2 - P.u3, P.f3);
+    const bool degen = rmul(0.5f, bn2) < lim;
+    const float ssl = degen ? sm : rfma(-abn, q.x, sm);
+    const float ssr = degen ? sm : rfma(abn, q.y, sm);
+    const float2 f1 = make_float2(P.f1.x, SPLIT ? P.f1.y : rfma(-bn, bn, P.f1t.y));
+    const float2 g1 = fma2(S, d1, f1);
+    const float2 g2 = fma2(S, fma2(P.nrho, v1, rs * v1s), P.f2);
+    const float2 g3 = fma2(S, fma2(P.nrho, v2, rs * v2s), P.f3);
     const float2 g4 = fma2(S, es - P.e, P.f4);
     const float2 g5 = fma2(S, b1s - b1, P.f5), g6 = fma2(S, b2s - b2, P.f6);
     // region 1 (*L), 2 (**L), 3 (**R), 4 (*R)
     const bool star_l = ssl >= 0.0f, left = star_l || sm >= 0.0f;
     const bool dbl = !star_l && (left || ssr >= 0.0f);
-    f[0] = left ? g0.x : g0.y;
-    f[1] = (left ? g1.x : g1.y) + ld1;
-    float h2 = left ? g2.x : g2.y, h3 = left ? g3.x : g3.y;
-    float h4 = fmaf(ld1, sm, left ? g4.x : g4.y);
-    float h5 = left ? g5.x : g5.y, h6 = left ? g6.x : g6.y;
+    f[0] = pick(left, g0);
+    f[1] = LD ? radd(pick(left, g1), pd) : pick(left, g1);
+    float h2 = pick(left, g2), h3 = pick(left, g3);
+    float h4 = LD ? rfma(pd, sm, pick(left, g4)) : pick(left, g4);
+    float h5 = pick(left, g5), h6 = pick(left, g6);
     if (dbl) {
       // double-star states: shared velocity and field, sqrt(rho*) weighted
       const float sgn = bn > 0.0f ? 1.0f : (bn < 0.0f ? -1.0f : 0.0f);
-      const float inv = rcp_(sq.x + sq.y), si = sgn * inv, qq = sq.x * sq.y * si;
-      const float wl = sq.x * inv, wr = sq.y * inv;
-      const float v1ss = fmaf(wl, v1s.x, fmaf(wr, v1s.y, (b1s.y - b1s.x) * si));
-      const float v2ss = fmaf(wl, v2s.x, fmaf(wr, v2s.y, (b2s.y - b2s.x) * si));
-      const float b1ss = fmaf(wl, b1s.y, fmaf(wr, b1s.x, (v1s.y - v1s.x) * qq));
-      const float b2ss = fmaf(wl, b2s.y, fmaf(wr, b2s.x, (v2s.y - v2s.x) * qq));
-      const float vbss = fmaf(v2ss, b2ss, fmaf(v1ss, b1ss, sm * bn));
-      const float r = left ? rs.x : rs.y, st = left ? ssl : ssr;
-      const float w = (left ? -sgn : sgn) * (left ? sq.x : sq.y);
-      const float d1 = v1ss - (left ? v1s.x : v1s.y), d2 = v2ss - (left ? v2s.x : v2s.y);
+      const float inv = recip(radd(sq.x, sq.y)), qq = rmul(sq.x, sq.y);
+      const float v1ss = rmul(rfma(rsub(b1s.y, b1s.x), sgn, rfma(sq.x, v1s.x, rmul(sq.y, v1s.y))), inv);
+      const float v2ss = rmul(rfma(rsub(b2s.y, b2s.x), sgn, rfma(sq.x, v2s.x, rmul(sq.y, v2s.y))), inv);
+      const float b1ss = rmul(rfma(rmul(qq, rsub(v1s.y, v1s.x)), sgn,
+                                   rfma(sq.x, b1s.y, rmul(sq.y, b1s.x))), inv);
+      const float b2ss = rmul(rfma(rmul(qq, rsub(v2s.y, v2s.x)), sgn,
+                                   rfma(sq.x, b2s.y, rmul(sq.y, b2s.x))), inv);
+      const float vbss = rfma(v2ss, b2ss, rfma(v1ss, b1ss, smb));
+      const float r = pick(left, rs), st = left ? ssl : ssr, ese = pick(left, es);
+      const float w = left ? -sq.x : sq.y;
+      const float ess = rfma(rmul(w, rsub(pick(left, vbs), vbss)), sgn, ese);
       // F** = F* + S* (U** - U*); rho** = rho* and u** = S_M
-      h2 = fmaf(st * r, d1, h2);
-      h3 = fmaf(st * r, d2, h3);
-      h4 = fmaf(st * w, (left ? vbs.x : vbs.y) - vbss, h4);
-      h5 = fmaf(st, b1ss - (left ? b1s.x : b1s.y), h5);
-      h6 = fmaf(st, b2ss - (left ? b2s.x : b2s.y), h6);
+      h2 = rfma(st, rfma(r, v1ss, -rmul(r, pick(left, v1s))), h2);
+      h3 = rfma(st, rfma(r, v2ss, -rmul(r, pick(left, v2s))), h3);
+      h4 = rfma(st, rsub(ess, ese), h4);
+      h5 = rfma(st, rsub(b1ss, pick(left, b1s)), h5);
+      h6 = rfma(st, rsub(b2ss, pick(left, b2s)), h6);
     }
     f[2] = h2; f[3] = h3; f[4] = h4; f[5] = h5; f[6] = h6;
   }
 }
 
-// HLLE (hlle of common.cuh) and the isothermal HLLE (g = cs^2, no energy):
-// F = (b+ F_L - b- F_R + b+ b- (U_R - U_L)) / (b+ - b-) as two packed
-// products a component and one sum of the halves.
-template <bool MHD, bool ISO>
-__device__ __forceinline__ void hlle2(float g, float igm1, const float2* W, float bn, float* f) {
-  const SidePair<MHD, ISO> P(g, igm1, W, bn, bn * bn);
-  const float2 un = W[1];
-  const float cm = fmaxf(P.cf.x, P.cf.y);
-  const float bm = fminf(fminf(un.x, un.y) - cm, 0.0f), bp = fmaxf(fmaxf(un.x, un.y) + cm, 0.0f);
-  const float inv = rcp_(bp - bm), c = bp * bm * inv;
-  const float2 wf = make_float2(bp * inv, -bm * inv), wu = make_float2(-c, c);
-  auto mix = [&](float2 fx, float2 u) {
-    const float2 t = fma2(wu, u, wf * fx);
-    return t.x + t.y;
-  };
-  f[0] = mix(P.f0, W[0]);
-  f[1] = mix(P.f1, P.f0);
-  f[2] = mix(P.f2, P.u2);
-  f[3] = mix(P.f3, P.u3);
-  f[4] = 0.0f;
-  if constexpr (!ISO) f[4] = mix(P.f4, P.e);
-  f[5] = f[6] = 0.0f;
-  if constexpr (MHD) {
-    f[5] = mix(P.f5, W[5]);
-    f[6] = mix(P.f6, W[6]);
-  }
-}
-
-// Isothermal HLLD (hlld_iso of common.cuh), g = cs^2.
-template <bool MHD>
+// Isothermal HLLD (hlld_iso of common.cuh), g = cs^2.  SPLIT: the right side's
+// induction fluxes are differences of two rounded products.
+template <bool MHD, bool SPLIT>
 __device__ __forceinline__ void hlld_iso2(float g, const float2* W, float bn, float* f) {
-  const float bn2 = bn * bn;
-  const SidePair<MHD, true> P(g, 0.0f, W, bn, bn2);
+  const float bn2 = rmul(bn, bn);
+  SidePair<MHD, true> P(g, 0.0f, W, bn, bn2);
   const float2 rho = W[0], un = W[1], v1 = W[2], v2 = W[3], b1 = W[5], b2 = W[6];
+  if constexpr (MHD && SPLIT) {
+    P.f5.y = rsub(rmul(b1.y, un.y), rmul(bn, v1.y));
+    P.f6.y = rsub(rmul(b2.y, un.y), rmul(bn, v2.y));
+  }
   const float cm = fmaxf(P.cf.x, P.cf.y);
-  const float2 S = make_float2(fminf(un.x, un.y) - cm, fmaxf(un.x, un.y) + cm);
+  const float2 S = make_float2(rsub(fminf(un.x, un.y), cm), radd(fmaxf(un.x, un.y), cm));
   f[4] = f[5] = f[6] = 0.0f;
   if (S.x >= 0.0f || S.y <= 0.0f) {
     const bool l = S.x >= 0.0f;
-    f[0] = l ? P.f0.x : P.f0.y;
-    f[1] = l ? P.f1.x : P.f1.y;
-    f[2] = l ? P.f2.x : P.f2.y;
-    f[3] = l ? P.f3.x : P.f3.y;
-    if constexpr (MHD) {
-      f[5] = l ? P.f5.x : P.f5.y;
-      f[6] = l ? P.f6.x : P.f6.y;
-    }
+    f[0] = pick(l, P.f0); f[1] = pick(l, P.f1); f[2] = pick(l, P.f2); f[3] = pick(l, P.f3);
+    if constexpr (MHD) { f[5] = pick(l, P.f5); f[6] = pick(l, P.f6); }
     return;
   }
-  const float idn = rcp_(S.y - S.x), ssp = S.x * S.y;
-  const float rs = (fmaf(S.y, rho.y, -S.x * rho.x) - (P.f0.y - P.f0.x)) * idn;
-  const float fm = fmaf(ssp, rho.y - rho.x, fmaf(S.y, P.f0.x, -S.x * P.f0.y)) * idn;
+  const float idn = recip(rsub(S.y, S.x)), ssp = rmul(S.x, S.y), df = rsub(P.f0.y, P.f0.x);
+  const float rs = rmul(rsub(rfma(S.y, rho.y, -rmul(S.x, rho.x)), df), idn);
+  const float fm = rmul(rfma(ssp, rsub(rho.y, rho.x), rfma(S.y, P.f0.x, -rmul(S.x, P.f0.y))), idn);
   f[0] = fm;
-  f[1] = fmaf(ssp, P.f0.y - P.f0.x, fmaf(S.y, P.f1.x, -S.x * P.f1.y)) * idn;
-  const float us = fm * rcp_(rs);
-  const float iq = rsqrtf(rs), sq = rs * iq, al = fabsf(bn) * iq;
-  const float ssl = us - al, ssr = us + al;
-  // transverse star states across the fast waves
-  const float2 su = S - un, m = rho * su, msu = m * su;
-  float2 v1s = v1, v2s = v2, b1s = b1, b2s = b2;
-  if constexpr (MHD) {
-    const float2 den = fma2(m, S - splat(us), splat(-bn2)), id = rcp2(den);
-    float2 nfv = (splat(bn) * id) * (un - splat(us)), fb = (msu - splat(bn2)) * id;
-    const float2 lim = (msu + splat(bn2)) * splat(Eps<float>::hlld);
+  f[1] = rmul(rfma(ssp, df, rfma(S.y, P.f1.x, -rmul(S.x, P.f1.y))), idn);
+  const float us = rmul(fm, recip(rs));
+  const float2 rs2 = splat(rs);
+  if constexpr (!MHD) {   // no Alfven waves: the side the flow comes from
+    const bool l = !(us < 0.0f);
+    f[2] = pick(l, fma2(S, fma2(rs2, v1, P.nrho * v1), P.f2));
+    f[3] = pick(l, fma2(S, fma2(rs2, v2, P.nrho * v2), P.f3));
+  } else {
+    const float sq = sqrtf(rs), isq = recip(sq), al = rmul(fabsf(bn), isq);
+    const float ssl = rsub(us, al), ssr = radd(us, al);
+    // transverse star states across the fast waves
+    const float2 su = S - un, m = rho * su;
+    const float2 den = fma2(m, S - splat(us), splat(-bn2));
+    const float2 id = make_float2(recip(den.x), recip(den.y));
+    float2 nfv = (splat(bn) * (un - splat(us))) * id, fb = (mul_apart(m, su) - splat(bn2)) * id;
+    const float2 lim = splat(Eps<float>::hlld) * fma2(m, su, splat(bn2));
     if (!(fabsf(den.x) >= lim.x)) { nfv.x = 0.0f; fb.x = 1.0f; }
     if (!(fabsf(den.y) >= lim.y)) { nfv.y = 0.0f; fb.y = 1.0f; }
-    v1s = fma2(b1, nfv, v1);
-    v2s = fma2(b2, nfv, v2);
-    b1s = b1 * fb;
-    b2s = b2 * fb;
-  }
-  const float2 rs2 = splat(rs);
-  const float2 g2 = fma2(S, rs2 * v1s - P.u2, P.f2);
-  const float2 g3 = fma2(S, rs2 * v2s - P.u3, P.f3);
-  const bool right = ssl < 0.0f && ssr <= 0.0f, central = ssl < 0.0f && ssr > 0.0f;
-  float h2 = right ? g2.y : g2.x, h3 = right ? g3.y : g3.x, h5 = 0.0f, h6 = 0.0f;
-  if constexpr (MHD) {
+    const float2 v1s = fma2(b1, nfv, v1), v2s = fma2(b2, nfv, v2), b1s = b1 * fb, b2s = b2 * fb;
+    const float2 g2 = fma2(S, fma2(rs2, v1s, P.nrho * v1), P.f2);
+    const float2 g3 = fma2(S, fma2(rs2, v2s, P.nrho * v2), P.f3);
     const float2 g5 = fma2(S, b1s - b1, P.f5), g6 = fma2(S, b2s - b2, P.f6);
-    h5 = right ? g5.y : g5.x;
-    h6 = right ? g6.y : g6.x;
-  }
-  if (central) {
-    // central state between the Alfven waves (equal densities both sides)
-    const float sgn = bn > 0.0f ? 1.0f : (bn < 0.0f ? -1.0f : 0.0f);
-    const float hv = 0.5f * sgn * iq, hb = 0.5f * sgn * sq, sr = ssl * rs;
-    float c1 = 0.5f * (v1s.y - v1s.x), c2 = 0.5f * (v2s.y - v2s.x);   // v** - v*_L
-    if constexpr (MHD) {
-      const float k1 = fmaf(hb, v1s.y - v1s.x, 0.5f * (b1s.y - b1s.x));   // B** - B*_L
-      const float k2 = fmaf(hb, v2s.y - v2s.x, 0.5f * (b2s.y - b2s.x));
-      c1 = fmaf(hv, b1s.y - b1s.x, c1);
-      c2 = fmaf(hv, b2s.y - b2s.x, c2);
-      h5 = fmaf(ssl, k1, h5);
-      h6 = fmaf(ssl, k2, h6);
+    const bool l = !(ssl < 0.0f && ssr <= 0.0f);
+    float h2 = pick(l, g2), h3 = pick(l, g3), h5 = pick(l, g5), h6 = pick(l, g6);
+    if (ssl < 0.0f && ssr > 0.0f) {
+      // central state between the Alfven waves (equal densities both sides)
+      const float sgn = bn > 0.0f ? 1.0f : (bn < 0.0f ? -1.0f : 0.0f), hs = rmul(0.5f, sq);
+      auto cv = [&](float2 v, float2 b) {
+        return rfma(0.5f, radd(v.x, v.y), rmul(rmul(rmul(0.5f, rsub(b.y, b.x)), sgn), isq));
+      };
+      auto cb = [&](float2 v, float2 b) {
+        return rfma(0.5f, radd(b.x, b.y), rmul(rmul(hs, rsub(v.y, v.x)), sgn));
+      };
+      h2 = rfma(ssl, rfma(rs, cv(v1s, b1s), -rmul(rs, v1s.x)), h2);
+      h3 = rfma(ssl, rfma(rs, cv(v2s, b2s), -rmul(rs, v2s.x)), h3);
+      h5 = rfma(ssl, rsub(cb(v1s, b1s), b1s.x), h5);
+      h6 = rfma(ssl, rsub(cb(v2s, b2s), b2s.x), h6);
     }
-    h2 = fmaf(sr, c1, h2);
-    h3 = fmaf(sr, c2, h3);
+    f[2] = h2; f[3] = h3; f[5] = h5; f[6] = h6;
   }
-  f[2] = h2; f[3] = h3; f[5] = h5; f[6] = h6;
 }
 
 }  // namespace aeth
