@@ -4,17 +4,28 @@
 // one pressureless Rusanov flux pass per direction for all species; then one
 // fused kernel that forms the explicit stage combination and solves the
 // implicit drag of every cell in closed form (arrowhead system, O(N) per
-// velocity component) in FP64, whatever the transport precision.
+// velocity component) in FP64 by default (aeth_config.drag_precision),
+// whatever the transport precision.
 //
-// The stage combinations run in the working precision; the drag solve runs
-// in FP64 by default (aeth_config.drag_precision) and its few divisions are
-// hoisted: 1/rho_k and 1/(1 + a_k) per species, one 1/den per cell.
+// The stage combinations run in the working precision.  GB300 executes an FP64
+// operation at 1/64 of the FP32 rate, and the solve's ~215 operations and ~65
+// conversions a cell made the update 68% of the step, so FP32 transport solves
+// in FP32 pairs (dfloat.cuh, about 48 bits: the same FP32 results but for rare
+// last bits; error against FP64 of 10 steps unchanged, 1.4e-7).  128^3, 8
+// species: the update 1751 -> 458 / 565 us a launch (1.6 and 2.2 GB: now bound
+// by memory latency at 16 warps an SM), the step 5169 -> 2504 us; 61 x 100 x 37,
+// 3 species, per-species precision: 395 -> 273 us a step.  The FP64 solve stays
+// for FP64 transport, the constant-coefficient law, and cells or constants
+// outside the pairs' range.
 //
 // IMEX2P with implicit weight g = 1 + 1/sqrt 2 and explicit weight
 // d = 1 - 1/(2g) in two registers (A, B):
 //   stage 2: X = U^n + g dt L(U^n), W = U^n + d dt L(U^n), U2 = drag_h(X),
 //            B <- U2, A <- W + (1-g)/g (U2 - X)          [(U2-X)/g = dt R(U2)]
 //   stage 3: Y = A + (1-d) dt L(U2), A <- drag_h(Y)      (h = g dt)
+#include <type_traits>
+
+#include "dfloat.cuh"
 #include "runtime.hpp"
 
 namespace aeth {
@@ -101,11 +112,106 @@ struct DustUpd {
   R dfloor;
 };
 
+// Bounds of the densities, momenta and implicit weights that the FP32 pairs take:
+// the low halves of their products stay above the smallest normal number
+// (what overflows shows in the sum of the drift energies).
+constexpr double kPairLo = 1e-10, kPairHi = 1e10;
+
+// The implicit drag of one cell in FP32 pairs: X = (gx, dx) -> (gy, dy), the
+// formulas of k_dust_update.  wide: the species solved in pairs (constants in
+// ak, ia, wk); the others in FP32 (fak, fia, fwk), their part of the gas sums
+// added to the pairs.  Returns false where a product overflowed.
+template <int NDMAX, bool SEL>
+__device__ __forceinline__ bool drag_pairs(const float* gx, const float (*dx)[4], int nd,
+                                           const dfloat* ak, const dfloat* ia, const dfloat* wk,
+                                           const float* fak, const float* fia, const float* fwk,
+                                           unsigned wide, int iso, float* gy, float (*dy)[4]) {
+  dfloat den(gx[0]);
+#pragma unroll
+  for (int s = 0; s < NDMAX; ++s) {
+    if (s >= nd) break;
+    if (!SEL || ((wide >> s) & 1u)) den = den + wk[s] * dx[s][0];
+    else den = den + dx[s][0] * fwk[s];
+  }
+  const dfloat inv = reciprocal(den);
+  dfloat dke2(0.0f);   // twice the change of the dust kinetic energy
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    dfloat num(gx[1 + q]);
+#pragma unroll
+    for (int s = 0; s < NDMAX; ++s) {
+      if (s >= nd) break;
+      if (!SEL || ((wide >> s) & 1u)) num = num + wk[s] * dx[s][1 + q];
+      else num = num + fwk[s] * dx[s][1 + q];
+    }
+    const dfloat vg = num * inv;
+    gy[1 + q] = (float)(vg * gx[0]);
+    const float vgf = (float)vg;
+#pragma unroll
+    for (int s = 0; s < NDMAX; ++s) {
+      if (s >= nd) break;
+      const float m0 = dx[s][1 + q], rk = dx[s][0];
+      if (!SEL || ((wide >> s) & 1u)) {
+        const dfloat m1 = ((ak[s] * rk) * vg + m0) * ia[s];
+        dy[s][1 + q] = (float)m1;
+        dke2 = dke2 + ((m1 + (-m0)) * (m1 + m0)) * reciprocal(dfloat(rk));
+      } else {
+        const float m1 = (m0 + rk * fak[s] * vgf) * fia[s];
+        dy[s][1 + q] = m1;
+        dke2 = dke2 + (m1 - m0) * (m1 + m0) * (1.0f / rk);
+      }
+    }
+  }
+  // total energy conserved: drift energy becomes gas heat (the isothermal
+  // closure carries its energy slot unchanged)
+  gy[4] = iso ? gx[4] : (float)(dke2 * -0.5f + gx[4]);
+  return fabsf(dke2.h) < 1e37f;
+}
+
+// The same in FP64 for the cells the pairs do not take: species with no
+// density (rho_k <= 0) keep their kinetic energy out of the balance.
+template <int NDMAX, bool SEL>
+__device__ __noinline__ void drag_far(const float* gx, const float (*dx)[4], int nd,
+                                      const double* ak, const double* ia, const double* wk,
+                                      const float* fak, const float* fia, const float* fwk,
+                                      unsigned wide, int iso, float* gy, float (*dy)[4]) {
+  const double rg = gx[0];
+  double den = rg;
+  for (int s = 0; s < nd; ++s)
+    den += !SEL || ((wide >> s) & 1u) ? (double)dx[s][0] * wk[s] : (double)(dx[s][0] * fwk[s]);
+  const double inv_den = 1.0 / den;
+  double dke2 = 0.0;
+  for (int q = 0; q < 3; ++q) {
+    double num = gx[1 + q];
+    for (int s = 0; s < nd; ++s)
+      num += !SEL || ((wide >> s) & 1u) ? wk[s] * (double)dx[s][1 + q]
+                                        : (double)(fwk[s] * dx[s][1 + q]);
+    const double vg = num * inv_den;
+    gy[1 + q] = (float)(rg * vg);
+    const float vgf = (float)vg;
+    for (int s = 0; s < nd; ++s) {
+      if (!SEL || ((wide >> s) & 1u)) {
+        const double rk = dx[s][0], m0 = dx[s][1 + q];
+        const double m1 = (m0 + rk * ak[s] * vg) * ia[s];
+        dy[s][1 + q] = (float)m1;
+        if (rk > 0.0) dke2 += (m1 - m0) * (m1 + m0) / rk;
+      } else {
+        const float rk = dx[s][0], m0 = dx[s][1 + q];
+        const float m1 = (m0 + rk * fak[s] * vgf) * fia[s];
+        dy[s][1 + q] = m1;
+        if (rk > 0.0f) dke2 += (double)((m1 - m0) * (m1 + m0) * (1.0f / rk));
+      }
+    }
+  }
+  gy[0] = gx[0];
+  gy[4] = iso ? gx[4] : (float)((double)gx[4] - 0.5 * dke2);
+}
+
 // Stage combination in the working precision R, implicit drag in DT.
-// SEL (DT = double, R = float): per-species precision -- the species whose
-// implicit weight a_k = h / t_k exceeds sel_ratio are solved in FP64, the
+// SEL (DT = dfloat, R = float): per-species precision -- the species whose
+// implicit weight a_k = h / t_k exceeds sel_ratio are solved in pairs, the
 // others in FP32; the gas sums over species (the denominator, the momentum
-// numerators and the drag heating) accumulate in FP64.
+// numerators and the drag heating) accumulate in pairs.
 // COEFF: the constant-coefficient drag law (drag_c = K_k, a_k = h K_k /
 // rho_k per cell).  iso: isothermal gas, whose energy slot takes no drag
 // heating.
@@ -118,24 +224,41 @@ __global__ void __launch_bounds__(256)
   __shared__ DT s_ak[NDMAX], s_ia[NDMAX], s_wk[NDMAX];
   __shared__ float f_ak[SEL ? NDMAX : 1], f_ia[SEL ? NDMAX : 1], f_wk[SEL ? NDMAX : 1];
   __shared__ unsigned s_wide;   // SEL: bit s set = species s in FP64
+  // PAIR: the FP64 solve in FP32 pairs; the FP64 constants stay for the cells
+  // outside the pairs' range
+  constexpr bool PAIR = std::is_same_v<DT, dfloat>;
+  __shared__ double w_ak[PAIR ? NDMAX : 1], w_ia[PAIR ? NDMAX : 1], w_wk[PAIR ? NDMAX : 1];
+  __shared__ int s_far;         // PAIR: a constant outside the pairs' range
   {
+    using CT = std::conditional_t<PAIR, double, DT>;
     const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
     if (SEL && tid == 0) s_wide = 0u;
+    if (PAIR && tid == 0) s_far = 0;
     __syncthreads();
     if (tid < nd && tid < NDMAX) {
-      const DT h = (DT)kImexG * (DT)(*A.dt);
-      const DT a = h * (DT)A.drag_c[tid];
-      const DT ia = DT(1) / (DT(1) + a);
-      s_ak[tid] = a;
-      s_ia[tid] = ia;
-      s_wk[tid] = a * ia;
+      const CT h = (CT)kImexG * (CT)(*A.dt);
+      const CT a = h * (CT)A.drag_c[tid];
+      const CT ia = CT(1) / (CT(1) + a);
+      if constexpr (PAIR) {
+        w_ak[tid] = a;
+        w_ia[tid] = ia;
+        w_wk[tid] = a * ia;
+        s_ak[tid] = dfloat::of(a);
+        s_ia[tid] = dfloat::of(ia);
+        s_wk[tid] = dfloat::of(a * ia);
+        if (!(a > kPairLo && a < kPairHi)) s_far = 1;
+      } else {
+        s_ak[tid] = a;
+        s_ia[tid] = ia;
+        s_wk[tid] = a * ia;
+      }
       if constexpr (SEL) {
         const float af = (float)h * (float)A.drag_c[tid];
         const float iaf = 1.0f / (1.0f + af);
         f_ak[tid] = af;
         f_ia[tid] = iaf;
         f_wk[tid] = af * iaf;
-        if (a > (DT)sel_ratio) atomicOr(&s_wide, 1u << tid);
+        if (a > (CT)sel_ratio) atomicOr(&s_wide, 1u << tid);
       }
     }
     __syncthreads();
@@ -186,8 +309,46 @@ __global__ void __launch_bounds__(256)
   // 1/rho_k and 1/den come from one division (simultaneous inversion,
   // Montgomery 1987: prefix products, one reciprocal, back-substitution).
   R gy[5], dy[NDMAX][4];
-  const DT rg = gx[0];
   gy[0] = gx[0];
+  if constexpr (PAIR) {
+    // FP32 pairs hold the solve to about 48 bits, the results rounded to FP32
+    // as from FP64, where no product leaves the FP32 exponent range; cells (or
+    // constants) outside these bounds, without density or not finite are
+    // solved in FP64
+    bool far = s_far || !(gx[0] > (R)kPairLo && gx[0] < (R)kPairHi);
+#pragma unroll
+    for (int q = 1; q < 5; ++q) far = far || !(fabsf(gx[q]) < (float)kPairHi);
+#pragma unroll
+    for (int s = 0; s < NDMAX; ++s) {
+      if (s >= nd) break;
+      dy[s][0] = dx[s][0];
+      far = far || !(dx[s][0] > (R)kPairLo && dx[s][0] < (R)kPairHi);
+#pragma unroll
+      for (int q = 1; q < 4; ++q) far = far || !(fabsf(dx[s][q]) < (float)kPairHi);
+    }
+    if (!far)
+      far = !drag_pairs<NDMAX, SEL>(gx, dx, nd, s_ak, s_ia, s_wk, f_ak, f_ia, f_wk,
+                                   SEL ? s_wide : ~0u, iso, gy, dy);
+    if (far) {
+      // rare: the arrays go through memory here only
+      float tg[5], td[NDMAX][4], og[5], od[NDMAX][4];
+#pragma unroll
+      for (int v = 0; v < 5; ++v) tg[v] = gx[v];
+#pragma unroll
+      for (int s = 0; s < NDMAX; ++s)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) td[s][q] = s < nd ? dx[s][q] : 0.0f;
+      drag_far<NDMAX, SEL>(tg, td, nd, w_ak, w_ia, w_wk, f_ak, f_ia, f_wk, SEL ? s_wide : ~0u, iso,
+                           og, od);
+#pragma unroll
+      for (int v = 0; v < 5; ++v) gy[v] = og[v];
+#pragma unroll
+      for (int s = 0; s < NDMAX; ++s)
+#pragma unroll
+        for (int q = 1; q < 4; ++q) dy[s][q] = od[s][q];
+    }
+  } else {
+    const DT rg = gx[0];
   if constexpr (COEFF) {
     // constant-coefficient law (Sec. 2.2): t_k = rho_k / K_k with the
     // stage's dust density, which the drag leaves unchanged, so the weight
@@ -225,60 +386,6 @@ __global__ void __launch_bounds__(256)
         const DT m1 = (m0 + rk[s] * ak[s] * vg) * ia[s];
         dy[s][1 + q] = (R)m1;
         dke2 += (m1 - m0) * (m1 + m0) * irk[s];
-      }
-    }
-    gy[4] = iso ? gx[4] : (R)((DT)gx[4] - DT(0.5) * dke2);
-  } else if constexpr (SEL) {
-    // per-species precision: FP64 for the stiff species (s_wide), FP32 for
-    // the rest; one FP64 division for the denominator, reciprocals of the
-    // densities in each species' own precision
-    const unsigned wide = s_wide;
-    DT den = rg;
-    DT ir64[NDMAX];    // 1 / rho_k of the FP64 species (0 for rho_k <= 0)
-    float ir32[NDMAX]; // the same for the FP32 species
-#pragma unroll
-    for (int s = 0; s < NDMAX; ++s) {
-      if (s >= nd) break;
-      dy[s][0] = dx[s][0];
-      ir64[s] = DT(0);
-      ir32[s] = 0.0f;
-      if ((wide >> s) & 1u) {
-        den += (DT)dx[s][0] * s_wk[s];
-        if ((DT)dx[s][0] > DT(0)) ir64[s] = DT(1) / (DT)dx[s][0];
-      } else {
-        den += (DT)((float)dx[s][0] * f_wk[s]);
-        if ((float)dx[s][0] > 0.0f) ir32[s] = 1.0f / (float)dx[s][0];
-      }
-    }
-    const DT inv_den = DT(1) / den;
-    DT dke2 = 0;
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      DT num = gx[1 + q];
-#pragma unroll
-      for (int s = 0; s < NDMAX; ++s) {
-        if (s >= nd) break;
-        if ((wide >> s) & 1u) num += s_wk[s] * (DT)dx[s][1 + q];
-        else num += (DT)(f_wk[s] * (float)dx[s][1 + q]);
-      }
-      const DT vg = num * inv_den;
-      gy[1 + q] = (R)(rg * vg);
-      const float vgf = (float)vg;
-#pragma unroll
-      for (int s = 0; s < NDMAX; ++s) {
-        if (s >= nd) break;
-        const R r = dx[s][0];
-        if ((wide >> s) & 1u) {
-          const DT rk = r, m0 = dx[s][1 + q];
-          const DT m1 = (m0 + rk * s_ak[s] * vg) * s_ia[s];
-          dy[s][1 + q] = (R)m1;
-          dke2 += (m1 - m0) * (m1 + m0) * ir64[s];
-        } else {
-          const float rk = (float)r, m0 = (float)dx[s][1 + q];
-          const float m1 = (m0 + rk * f_ak[s] * vgf) * f_ia[s];
-          dy[s][1 + q] = (R)m1;
-          dke2 += (DT)((m1 - m0) * (m1 + m0) * ir32[s]);
-        }
       }
     }
     gy[4] = iso ? gx[4] : (R)((DT)gx[4] - DT(0.5) * dke2);
@@ -348,6 +455,7 @@ __global__ void __launch_bounds__(256)
   // total energy conserved: drift energy becomes gas heat (the isothermal
   // closure carries its energy slot unchanged)
   gy[4] = iso ? gx[4] : (R)((DT)gx[4] - dke);
+  }
   }
   int hits = 0;
 #pragma unroll
@@ -506,8 +614,14 @@ static void stage_dust(aeth_ctx* c, int b, int src, int stage) {
   if constexpr (sizeof(R) == 4) {
     if (c->cfg.drag_precision == AETH_DRAG_SEL64) {
       // per-species precision: FP64 for the species with h / t_k > drag_ratio
-      if (nd <= 8) launch(k_dust_update<R, double, 8, true>);
-      else launch(k_dust_update<R, double, 32, true>);
+      if (nd <= 8) launch(k_dust_update<R, dfloat, 8, true>);
+      else launch(k_dust_update<R, dfloat, 32, true>);
+      done = true;
+    } else if (d64 && !coeff) {
+      // FP32 transport with the FP64 drag: FP32 pairs
+      if (nd <= 4) launch(k_dust_update<R, dfloat, 4>);
+      else if (nd <= 8) launch(k_dust_update<R, dfloat, 8>);
+      else launch(k_dust_update<R, dfloat, 32>);
       done = true;
     }
   }
@@ -517,10 +631,10 @@ static void stage_dust(aeth_ctx* c, int b, int src, int stage) {
                      : launch(k_dust_update<R, R, 8, false, true>);
     else d64 ? launch(k_dust_update<R, double, 32, false, true>)
              : launch(k_dust_update<R, R, 32, false, true>);
-  } else if (nd <= 8) {
-    d64 ? launch(k_dust_update<R, double, 8>) : launch(k_dust_update<R, R, 8>);
+  } else if (nd <= 8) {   // FP64 transport, or the drag in FP32
+    launch(k_dust_update<R, R, 8>);
   } else {
-    d64 ? launch(k_dust_update<R, double, 32>) : launch(k_dust_update<R, R, 32>);
+    launch(k_dust_update<R, R, 32>);
   }
   c->n_launch += 3 + 1;
 }
