@@ -145,7 +145,11 @@ __device__ __forceinline__ Quad<double> plm_half(const Quad<double>& m, const Qu
                                                  const Quad<double>& p) {
   Quad<double> t;
 #pragma unroll
-  for (int q = 0; q < 4; ++q) t.v[q] = 0.5 * vl_slope(m.v[q], c.v[q], p.v[q]);
+  for (int q = 0; q < 4; ++q) {
+    // half of 2 dm dp / (dm + dp): the factors are powers of two
+    const double dm = c.v[q] - m.v[q], dp = p.v[q] - c.v[q], x = dm * dp;
+    t.v[q] = is_pos(x) ? x / (dm + dp) : 0.0;
+  }
   return t;
 }
 
