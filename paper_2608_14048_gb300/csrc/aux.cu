@@ -3,6 +3,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "ghost.cuh"
 #include "runtime.hpp"
 
 namespace aeth {
@@ -237,69 +238,36 @@ aeth_status build_tables(aeth_ctx* c) {
 }
 
 // ------------------------------------------------------------------------
-// ghost fill, one axis at a time (edges and corners come out right)
+// ghost fill of one block's arrays (unfused path, dust gas, training samples)
 // ------------------------------------------------------------------------
 
 template <typename R>
-__global__ void k_fill_axis(Layout L, Arr8<R> a, int nv, int d) {
-  const int g = L.g;
-  int lo[3], ext[3];
-  for (int e = 0; e < 3; ++e) {
-    if (e < d) { lo[e] = -g; ext[e] = L.n[e] + 2 * g + 1; }
-    else if (e == d) { lo[e] = 0; ext[e] = 2 * g + 1; }
-    else { lo[e] = 0; ext[e] = L.n[e] + 1; }
-  }
-  const int t0 = blockIdx.x * blockDim.x + threadIdx.x;
-  const int t1 = blockIdx.y * blockDim.y + threadIdx.y;
-  const int t2 = blockIdx.z * blockDim.z + threadIdx.z;
-  if (t0 >= ext[0] || t1 >= ext[1] || t2 >= ext[2]) return;
-  int c[3] = {t0 + lo[0], t1 + lo[1], t2 + lo[2]};
-  const int n = L.n[d];
-  const int t = c[d];
-  c[d] = t < g ? t - g : n + (t - g);      // -g..-1, n..n+g
-  const int p = c[d];
+__global__ void __launch_bounds__(256) k_fill_one(Layout L, Arr8<R> a, int nv) {
+  const unsigned el = blockIdx.x * blockDim.x + threadIdx.x;
+  if (el >= (unsigned)ghost_cells(L)) return;
+  int c[3];
+  ghost_cell(L, el, c);
   const long long dst = L.idx(c[0], c[1], c[2]);
+  bool up[3];
+#pragma unroll
+  for (int e = 0; e < 3; ++e) c[e] = ghost_axis(L, e, c[e], up[e]);
+  const long long src = L.idx(c[0], c[1], c[2]);
   // every source loaded before the first store: the stores go through the
   // same arrays, so interleaving them would serialise the round trips
   R val[NVAR];
-  bool on[NVAR];
-#pragma unroll
-  for (int v = 0; v < NVAR; ++v) {
-    on[v] = false;
-    if (v >= nv) continue;
-    const bool face_d = (v == 5 + d);
-    int s;
-    if (L.bc[d] == AETH_BC_PERIODIC) {
-      s = ((p % n) + n) % n;
-    } else if (face_d) {
-      if (p >= 0 && p <= n) continue;       // faces 0..n are real
-      s = p < 0 ? 0 : n;
-    } else {
-      s = p < 0 ? 0 : n - 1;
-    }
-    int sc[3] = {c[0], c[1], c[2]};
-    sc[d] = s;
-    val[v] = a.p[v][L.idx(sc[0], sc[1], sc[2])];
-    on[v] = true;
-  }
 #pragma unroll
   for (int v = 0; v < NVAR; ++v)
-    if (on[v]) a.p[v][dst] = val[v];
+    if (v < nv) val[v] = a.p[v][v >= 5 && up[v - 5] ? src + L.stride(v - 5) : src];
+#pragma unroll
+  for (int v = 0; v < NVAR; ++v)
+    if (v < nv && !(v >= 5 && up[v - 5] && src + L.stride(v - 5) == dst)) a.p[v][dst] = val[v];
 }
 
 template <typename R>
 void launch_fill(const BlockPtrs<R>& P, R* const* arrs, int nv, cudaStream_t st) {
   Arr8<R> a{};
   for (int v = 0; v < nv; ++v) a.p[v] = arrs[v];
-  const Layout& L = P.L;
-  for (int d = 0; d < 3; ++d) {
-    int ext[3];
-    for (int e = 0; e < 3; ++e)
-      ext[e] = e < d ? L.n[e] + 2 * L.g + 1 : (e == d ? 2 * L.g + 1 : L.n[e] + 1);
-    dim3 blk(32, 4, 2);
-    dim3 grd((ext[0] + 31) / 32, (ext[1] + 3) / 4, (ext[2] + 1) / 2);
-    k_fill_axis<R><<<grd, blk, 0, st>>>(L, a, nv, d);
-  }
+  k_fill_one<R><<<ceil_div(ghost_cells(P.L), 256), 256, 0, st>>>(P.L, a, nv);
 }
 template void launch_fill<float>(const BlockPtrs<float>&, float* const*, int, cudaStream_t);
 template void launch_fill<double>(const BlockPtrs<double>&, double* const*, int, cudaStream_t);
@@ -477,6 +445,41 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// The end of a CFL pass: the CTA's minimum into partial[], and in the CTA that
+// arrives last (a counter that it sets back to zero) the minimum of all of
+// them, scaled, as the step.  A launch of its own for this cost 4 to 8 us.
+struct DtFinal {
+  unsigned* arrived;
+  double scale;
+  double* dt;
+};
+__device__ __forceinline__ void dt_reduce(double m, double* sm, double* partial, const DtFinal& f) {
+  __shared__ bool last;
+  auto block_min = [&](double v) {   // in thread 0
+    v = warp_min(v);
+    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x < 32) v = warp_min(threadIdx.x < (blockDim.x >> 5) ? sm[threadIdx.x] : INFINITY);
+    return v;
+  };
+  const double v = block_min(m);
+  if (threadIdx.x == 0) {
+    partial[blockIdx.x] = v;
+    __threadfence();
+    last = atomicAdd(f.arrived, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double all = INFINITY;
+  for (unsigned t = threadIdx.x; t < gridDim.x; t += blockDim.x) all = fmin(all, __ldcg(partial + t));
+  all = block_min(all);
+  if (threadIdx.x == 0) {
+    *f.dt = f.scale * all;
+    *f.arrived = 0u;
+  }
+}
+
 // CFL time step (Eq. 11) over all blocks: one partial minimum per CTA.  The
 // work unit is the 32x4x2 cell tile of the elementwise passes (full warps
 // on every block size, one block lookup per 256 cells); a CTA iteration
@@ -487,8 +490,8 @@ __device__ __forceinline__ double warp_sum(double v) {
 template <typename R, bool P64, typename Src, bool DUAL = false>
 __global__ void __launch_bounds__(256)
     k_dt(Src S, int total, int mhd, double gamma, double rho_floor, double p_floor, int nd,
-         double cs2, double alpha_switch, float p64_ratio, double* __restrict__ partial,
-         int* status) {
+         double cs2, double alpha_switch, float p64_ratio, double* partial,
+         int* status, DtFinal fin) {
   constexpr bool dual = DUAL;
   // cs2 > 0: isothermal closure p = cs2 rho, fast speed with gamma = 1
   const bool iso = cs2 > 0.0;
@@ -598,15 +601,8 @@ __global__ void __launch_bounds__(256)
       }
     }
   }
-  const double md = warp_min((double)m);
-  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = md;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double v = threadIdx.x < (blockDim.x >> 5) ? sm[threadIdx.x] : INFINITY;
-    v = warp_min(v);
-    if (threadIdx.x == 0) partial[blockIdx.x] = v;
-  }
   if (bad) atomicOr(status, ST_NONFINITE);
+  dt_reduce(m, sm, partial, fin);
 }
 
 // 0: the one-cell-per-thread CFL pass everywhere
@@ -630,7 +626,7 @@ __device__ __forceinline__ float el4(const float4& v, int q) {
 template <bool P64, typename Src>
 __global__ void __launch_bounds__(256)
     k_dt_v4(Src S, int total, int mhd, float gamma, float rho_floor, float p_floor, float cs2,
-            float p64_ratio, double* __restrict__ partial, int* status) {
+            float p64_ratio, double* partial, int* status, DtFinal fin) {
   __shared__ double sm[8];
   const bool iso = cs2 > 0.0f;
   float m = INFINITY;
@@ -722,30 +718,8 @@ __global__ void __launch_bounds__(256)
       cell(el4(r4, q), el4(a4, q), el4(b4, q), el4(c4, q), el4(e4, q), bc, wd);
     }
   }
-  const double md = warp_min((double)m);
-  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = md;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double v = threadIdx.x < (blockDim.x >> 5) ? sm[threadIdx.x] : INFINITY;
-    v = warp_min(v);
-    if (threadIdx.x == 0) partial[blockIdx.x] = v;
-  }
   if (bad) atomicOr(status, ST_NONFINITE);
-}
-
-__global__ void k_dt_final(const double* __restrict__ partial, int n, double scale,
-                           double* __restrict__ dt) {
-  __shared__ double sm[32];
-  double m = INFINITY;
-  for (int t = threadIdx.x; t < n; t += blockDim.x) m = fmin(m, partial[t]);
-  m = warp_min(m);
-  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = m;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double v = threadIdx.x < (blockDim.x >> 5) ? sm[threadIdx.x] : INFINITY;
-    v = warp_min(v);
-    if (threadIdx.x == 0) *dt = scale * v;
-  }
+  dt_reduce(m, sm, partial, fin);
 }
 
 template <typename R, bool P64>
@@ -756,8 +730,8 @@ static aeth_status dt_T(aeth_ctx* c) {
   const int grid = std::max(1, std::min(c->dt_grid, (total + 1) / 2));
   const double cs2 = is_iso(c) ? c->cfg.cs_iso * c->cfg.cs_iso : 0.0;
   const double dual_a = is_dual(c) ? c->cfg.alpha_switch : 0.0;
-  // returns the number of partial minima written
-  auto launch = [&](auto src) -> int {
+  const DtFinal fin{c->d_arrived, c->cfg.cfl * cmax_of(c->cfg.integrator), c->d_dt};
+  auto launch = [&](auto src) {
     using Src = decltype(src);
     if constexpr (sizeof(R) == 4) {
       if (dual_a <= 0.0 && c->cfg.n_dust == 0 && AETH_DT_V4) {
@@ -767,8 +741,8 @@ static aeth_status dt_T(aeth_ctx* c) {
             src, total, is_mhd(c), (float)c->cfg.gamma, (float)c->cfg.rho_floor,
             (float)c->cfg.p_floor, (float)cs2,
             c->cfg.precision == AETH_FP32_SEL64 ? (float)c->cfg.p64_ratio : 0.0f, c->d_partials,
-            c->d_status);
-        return g4;
+            c->d_status, fin);
+        return;
       }
     }
     auto kernel = dual_a > 0.0 ? k_dt<R, P64, Src, true> : k_dt<R, P64, Src, false>;
@@ -776,19 +750,15 @@ static aeth_status dt_T(aeth_ctx* c) {
                                          c->cfg.p_floor, c->cfg.n_dust, cs2, dual_a,
                                          c->cfg.precision == AETH_FP32_SEL64
                                              ? (float)c->cfg.p64_ratio : 0.0f,
-                                         c->d_partials, c->d_status);
-    return grid;
+                                         c->d_partials, c->d_status, fin);
   };
-  int nparts;
   if (nb == 1) {
-    nparts = launch(ParamSrc<R>{block_ptrs<R>(c, 0), 0});
+    launch(ParamSrc<R>{block_ptrs<R>(c, 0), 0});
   } else {
-    nparts = launch(TableSrc<R>{(const BlockPtrs<R>*)c->d_tab, c->d_prefix + PK_CELL * (nb + 1),
+    launch(TableSrc<R>{(const BlockPtrs<R>*)c->d_tab, c->d_prefix + PK_CELL * (nb + 1),
                                 nb, c->d_tmap[PK_CELL]});
   }
-  c->n_launch += 2;
-  const double scale = c->cfg.cfl * cmax_of(c->cfg.integrator);
-  k_dt_final<<<1, 1024, 0, c->stream>>>(c->d_partials, nparts, scale, c->d_dt);
+  c->n_launch += 1;
   AETH_CK(c, cudaGetLastError());
   return AETH_OK;
 }

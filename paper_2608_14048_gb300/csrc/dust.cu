@@ -26,6 +26,7 @@
 #include <type_traits>
 
 #include "dfloat.cuh"
+#include "ghost.cuh"
 #include "runtime.hpp"
 
 namespace aeth {
@@ -498,31 +499,18 @@ __global__ void __launch_bounds__(256)
   if (hits) atomicAdd(floor_hits, (unsigned long long)hits);
 }
 
-// Ghost fill of n cell-centred arrays at base + a * sz, one axis.
+// Ghost fill of narr cell-centred arrays at base + a * sz.
 template <typename R>
-__global__ void __launch_bounds__(256) k_fill_cells(Layout L, R* base, int narr, int d) {
-  const int g = L.g;
-  int lo[3], ext[3];
-  for (int e = 0; e < 3; ++e) {
-    if (e < d) { lo[e] = -g; ext[e] = L.n[e] + 2 * g + 1; }
-    else if (e == d) { lo[e] = 0; ext[e] = 2 * g + 1; }
-    else { lo[e] = 0; ext[e] = L.n[e] + 1; }
-  }
-  const int t0 = blockIdx.x * blockDim.x + threadIdx.x;
-  const int t1 = blockIdx.y * blockDim.y + threadIdx.y;
-  const int t2 = blockIdx.z * blockDim.z + threadIdx.z;
-  if (t0 >= ext[0] || t1 >= ext[1] || t2 >= ext[2]) return;
-  int c[3] = {t0 + lo[0], t1 + lo[1], t2 + lo[2]};
-  const int n = L.n[d];
-  const int t = c[d];
-  c[d] = t < g ? t - g : n + (t - g);
-  const int p = c[d];
-  int s;
-  if (L.bc[d] == AETH_BC_PERIODIC) s = ((p % n) + n) % n;
-  else s = p < 0 ? 0 : n - 1;
-  int sc[3] = {c[0], c[1], c[2]};
-  sc[d] = s;
-  const long long dst = L.idx(c[0], c[1], c[2]), srcx = L.idx(sc[0], sc[1], sc[2]);
+__global__ void __launch_bounds__(256) k_fill_cells(Layout L, R* base, int narr) {
+  const unsigned el = blockIdx.x * blockDim.x + threadIdx.x;
+  if (el >= (unsigned)ghost_cells(L)) return;
+  int c[3];
+  ghost_cell(L, el, c);
+  const long long dst = L.idx(c[0], c[1], c[2]);
+  bool up;
+#pragma unroll
+  for (int e = 0; e < 3; ++e) c[e] = ghost_axis(L, e, c[e], up);
+  const long long srcx = L.idx(c[0], c[1], c[2]);
   const long long sz = L.size();
   // eight arrays at a time, every source loaded before the stores (the
   // stores go through the same base, so interleaving them would serialise
@@ -546,17 +534,8 @@ static void stage_dust(aeth_ctx* c, int b, int src, int stage) {
   const int nd = c->cfg.n_dust;
   cudaStream_t s = c->stream;
   launch_fill<R>(P, P.reg[src], 5, s);
-  c->n_launch += 3;
-  const long long sz = L.size();
-  (void)sz;
-  for (int d = 0; d < 3; ++d) {
-    int ext[3];
-    for (int e = 0; e < 3; ++e)
-      ext[e] = e < d ? L.n[e] + 2 * L.g + 1 : (e == d ? 2 * L.g + 1 : L.n[e] + 1);
-    dim3 fb(32, 4, 2), fg((ext[0] + 31) / 32, (ext[1] + 3) / 4, (ext[2] + 1) / 2);
-    k_fill_cells<R><<<fg, fb, 0, s>>>(L, P.dust[src], 4 * nd, d);
-  }
-  c->n_launch += 3;
+  k_fill_cells<R><<<ceil_div(ghost_cells(L), 256), 256, 0, s>>>(L, P.dust[src], 4 * nd);
+  c->n_launch += 2;
   hydro_flux_pass<R, P64>(c, b, c->cfg.recon, src);
   dim3 blk(32, 4, 2);
   dim3 grd((L.n[0] + 1 + 31) / 32, (L.n[1] + 1 + 3) / 4, (L.n[2] + 1 + 1) / 2);

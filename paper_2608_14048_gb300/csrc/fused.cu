@@ -14,11 +14,9 @@
 //  3. k_update_f: finite-volume update (Eq. 8, curvilinear sources of
 //     Eq. 12) and constrained transport (Eq. 9) with the stage combination.
 #include "flux3.cuh"
+#include "ghost.cuh"
 
 namespace aeth {
-
-template <typename R>
-void launch_fill(const BlockPtrs<R>& P, R* const* arrs, int nv, cudaStream_t st);
 
 // resident CTAs per SM requested for the update pass (registers 65536 /
 // (256 * UPD_MINB)): the loads of a cell are hoisted above its stores, so
@@ -674,101 +672,90 @@ __global__ void __launch_bounds__(256) k_dual_sync(Src S, int t0, int t1, int re
 }
 
 // ------------------------------------------------------------------------
-// ghost fill of one register, one axis per launch (Sec. 2.3); LINKS and ENT
-// compile the linked-block and entropy copies in only where the context has
-// them (each costs registers in the plain fill)
+// ghost fill of one register (Sec. 2.3, ghost.cuh), threads linear over the
+// ghost cells of every block; LINKS and ENT compile the linked-block and
+// entropy copies in only where the context has them (each costs registers in
+// the plain fill)
 // ------------------------------------------------------------------------
 template <typename R, typename Src, bool LINKS, bool ENT>
-__global__ void __launch_bounds__(256) k_fill_b(Src S, int t0, int t1, int reg, int nv, int d) {
-  for (int t = t0 + (int)blockIdx.x; t < t1; t += gridDim.x) {
-    int loc;
-    const BlockPtrs<R>& B = S.get(t, loc);
-    const Layout L = B.L;
-    const int g = L.g;
-    int lo[3], ext[3];
-    for (int e = 0; e < 3; ++e) {
-      if (e < d) { lo[e] = -g; ext[e] = L.n[e] + 2 * g + 1; }
-      else if (e == d) { lo[e] = 0; ext[e] = 2 * g + 1; }
-      else { lo[e] = 0; ext[e] = L.n[e] + 1; }
-    }
-    // threads run linearly over the slab (x fastest): every lane busy even
-    // where the slab is only 2g+1 cells thick along x
-    const long long el = (long long)loc * FILL_TILE + threadIdx.x;
-    if (el >= (long long)ext[0] * ext[1] * ext[2]) continue;
-    const int t0c = (int)(el % ext[0]);
-    const int t1c = (int)((el / ext[0]) % ext[1]);
-    const int t2c = (int)(el / ((long long)ext[0] * ext[1]));
-    int c[3] = {t0c + lo[0], t1c + lo[1], t2c + lo[2]};
-    const int n = L.n[d];
-    const int tt = c[d];
-    c[d] = tt < g ? tt - g : n + (tt - g);
-    const int p = c[d];
-    const long long dst = L.idx(c[0], c[1], c[2]);
-    // a linked side copies from the neighbouring block's cells (and faces)
-    // beyond it: cells n_nb + p on the low side, p - n on the high side
-    const int lk = LINKS ? L.lnk[d][p < 0 ? 0 : 1] : -1;
-    const BlockPtrs<R>& SB = (lk < 0 || lk == L.self) ? B : B.tab[lk];
-    // every source is loaded before the first store (the stores go through
-    // pointer arrays the compiler cannot prove disjoint from the loads)
-    R val[NVAR];
-    bool on[NVAR];
+__global__ void __launch_bounds__(256) k_fill_b(Src S, int t0, int reg, int nv) {
+  int loc;
+  const BlockPtrs<R>& B = S.get(t0 + (int)blockIdx.x, loc);
+  const Layout& L = B.L;
+  const unsigned el = (unsigned)loc * FILL_TILE + threadIdx.x;
+  if (el >= (unsigned)ghost_cells(L)) return;
+  int c[3];
+  ghost_cell(L, el, c);
+  const long long dst = L.idx(c[0], c[1], c[2]);
+  // the axis maps in the order z, y, x, each in the block the previous one
+  // leads to: a linked side goes on in the neighbouring block (cells n_nb + p
+  // below, p - n above), as the fill axis by axis does
+  const BlockPtrs<R>* SB = &B;
+  bool up[3];
 #pragma unroll
-    for (int v = 0; v < NVAR; ++v) {
-      on[v] = false;
-      if (v >= nv) continue;
-      const bool face_d = (v == 5 + d);
-      int s;
-      if (lk >= 0) {
-        s = p < 0 ? SB.L.n[d] + p : p - n;
-      } else if (L.bc[d] == AETH_BC_PERIODIC) {
-        s = ((p % n) + n) % n;
-      } else if (face_d) {
-        if (p >= 0 && p <= n) continue;
-        s = p < 0 ? 0 : n;
-      } else {
-        s = p < 0 ? 0 : n - 1;
-      }
-      int sc[3] = {c[0], c[1], c[2]};
-      sc[d] = s;
-      val[v] = SB.reg[reg][v][SB.L.idx(sc[0], sc[1], sc[2])];
-      on[v] = true;
+  for (int e = 2; e >= 0; --e) {
+    int p = c[e];
+    // the second hop: index n + g over a neighbour of only g cells
+    for (int hop = 0; LINKS && hop < 2; ++hop) {
+      const int n = SB->L.n[e];
+      const int lk = p < 0 || p >= n ? SB->L.lnk[e][p < 0 ? 0 : 1] : -1;
+      if (lk < 0) break;
+      if (lk != SB->L.self) SB = B.tab + lk;
+      p = p < 0 ? SB->L.n[e] + p : p - n;
     }
-#pragma unroll
-    for (int v = 0; v < NVAR; ++v)
-      if (on[v]) B.reg[reg][v][dst] = val[v];
-    // dual energy: the entropy is a cell variable like the density
-    if constexpr (ENT) {
-      R* e = B.ent[reg];
-      int sc[3] = {c[0], c[1], c[2]};
-      if (lk >= 0) sc[d] = p < 0 ? SB.L.n[d] + p : p - n;
-      else sc[d] = L.bc[d] == AETH_BC_PERIODIC ? ((p % n) + n) % n : (p < 0 ? 0 : n - 1);
-      e[dst] = SB.ent[reg][SB.L.idx(sc[0], sc[1], sc[2])];
-    }
+    c[e] = ghost_axis(SB->L, e, p, up[e]);
   }
+  const long long src = SB->L.idx(c[0], c[1], c[2]);
+  // every source is loaded before the first store (the stores go through
+  // pointer arrays the compiler cannot prove disjoint from the loads)
+  R val[NVAR], ent = R(0);
+#pragma unroll
+  for (int v = 0; v < NVAR; ++v) {
+    if (v >= nv) continue;
+    const BlockPtrs<R>* FB = SB;
+    long long at = src;
+    if (v >= 5 && up[v - 5]) {
+      const int e = v - 5;
+      at += SB->L.stride(e);
+      // an outflow face n that a later link led into a block which goes on
+      // there: the same face is number 0 beyond it
+      const int lk = LINKS ? SB->L.lnk[e][1] : -1;
+      if (lk >= 0 || (LINKS && SB->L.bc[e] == AETH_BC_PERIODIC)) {
+        if (lk >= 0 && lk != SB->L.self) FB = B.tab + lk;
+        at = FB->L.idx(e == 0 ? 0 : c[0], e == 1 ? 0 : c[1], e == 2 ? 0 : c[2]);
+      }
+    }
+    val[v] = FB->reg[reg][v][at];
+  }
+  if constexpr (ENT) ent = SB->ent[reg][src];
+#pragma unroll
+  for (int v = 0; v < NVAR; ++v)
+    if (v < nv) {
+      // face n of an outflow axis is real: not a copy of itself
+      if (v >= 5 && up[v - 5] && SB == &B && src + L.stride(v - 5) == dst) continue;
+      B.reg[reg][v][dst] = val[v];
+    }
+  if constexpr (ENT) B.ent[reg][dst] = ent;   // a cell variable like the density
 }
 
 // ------------------------------------------------------------------------
 // host side
 // ------------------------------------------------------------------------
 template <typename R, bool LINKS, bool ENT>
-static void launch_fill_axes(aeth_ctx* c, int reg, int nv, int block) {
-  for (int d = 0; d < 3; ++d) {
-    with_src<R>(c, PK_FILL0 + d, block, [&](auto S, TileRange r) {
-      if (r.t1 <= r.t0) return;
-      k_fill_b<R, decltype(S), LINKS, ENT><<<r.t1 - r.t0, 256, 0, c->stream>>>(S, r.t0, r.t1,
-                                                                               reg, nv, d);
-    });
-  }
-  c->n_launch += 3;
+static void launch_fill_b(aeth_ctx* c, int reg, int nv, int block) {
+  with_src<R>(c, PK_FILL, block, [&](auto S, TileRange r) {
+    k_fill_b<R, decltype(S), LINKS, ENT><<<r.t1 - r.t0, 256, 0, c->stream>>>(S, r.t0, reg, nv);
+  });
+  c->n_launch += 1;
 }
 
 template <typename R>
 static void launch_fill_all(aeth_ctx* c, int reg, int nv, int block) {
   const bool links = !c->links.empty(), ent = is_dual(c);
-  if (links && ent) launch_fill_axes<R, true, true>(c, reg, nv, block);
-  else if (links) launch_fill_axes<R, true, false>(c, reg, nv, block);
-  else if (ent) launch_fill_axes<R, false, true>(c, reg, nv, block);
-  else launch_fill_axes<R, false, false>(c, reg, nv, block);
+  if (links && ent) launch_fill_b<R, true, true>(c, reg, nv, block);
+  else if (links) launch_fill_b<R, true, false>(c, reg, nv, block);
+  else if (ent) launch_fill_b<R, false, true>(c, reg, nv, block);
+  else launch_fill_b<R, false, false>(c, reg, nv, block);
 }
 
 template <typename R>

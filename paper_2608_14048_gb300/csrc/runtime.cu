@@ -282,7 +282,7 @@ aeth_status aeth_plan(aeth_ctx* c, size_t* bytes) {
   off += align256((size_t)PK_N * (nb + 1) * sizeof(int));
   for (int kind = 0; kind < PK_N; ++kind) {
     c->tmap_n[kind] = 0;
-    if (nb < 2 || !(kind == PK_CELL || (kind >= PK_FILL0 && kind <= PK_FILL2))) continue;
+    if (nb < 2 || !(kind == PK_CELL || kind == PK_FILL)) continue;
     long long tiles = 0;
     for (const auto& B : c->blocks) tiles += tiles_of(B.L, kind, 0);
     c->off_tmap[kind] = off;
@@ -326,6 +326,7 @@ aeth_status aeth_finalize(aeth_ctx* c, size_t* bytes) {
   char* sc = c->arena + c->off_scalars;
   c->d_dt = (double*)sc;
   c->d_diag = (double*)(sc + 64);
+  c->d_arrived = (unsigned*)(sc + 192);
   c->d_status = (int*)(sc + 256);
   c->d_floor = (unsigned long long*)(sc + 320);
   c->d_fallback = (unsigned long long*)(sc + 384);

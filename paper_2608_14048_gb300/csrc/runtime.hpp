@@ -51,8 +51,7 @@ struct BlockInfo {
 
 // Pass kinds of the batched launches; each has a prefix sum of tiles per
 // mesh block so that one launch covers every block.
-enum PassKind : int { PK_FLUX = 0, PK_CELL = 1, PK_FILL0 = 2, PK_FILL1 = 3, PK_FILL2 = 4,
-                      PK_ROWS = 5, PK_N = 6 };
+enum PassKind : int { PK_FLUX = 0, PK_CELL = 1, PK_FILL = 2, PK_ROWS = 3, PK_N = 4 };
 
 // Tile geometry of each pass kind (threads per tile fixed per kind).
 // 2-D flux tiles: 128 threads, FLUX_TX x (FLUX_NT / FLUX_TX) by default
@@ -78,10 +77,16 @@ constexpr int FILL_TILE = 256;   // ghost cells per tile of the fill pass
 
 inline int ceil_div(long long a, long long b) { return (int)((a + b - 1) / b); }
 
+// Cells of the padded array (index -g to n + g on each axis) outside the
+// interior.
+__host__ __device__ inline long long ghost_cells(const Layout& L) {
+  const long long T = 2 * L.g + 1, X = L.n[0] + T, Y = L.n[1] + T;
+  return T * X * Y + L.n[2] * T * X + (long long)L.n[2] * L.n[1] * T;
+}
+
 // Tiles of one block for a pass kind (kchunk: z extent of a flux tile,
 // tx: its x width, FLUX_NT / tx its y width; tx = 0: band tiles).
 inline int tiles_of(const Layout& L, int kind, int kchunk, int tx = FLUX_TX) {
-  const int g = L.g;
   if (kind == PK_FLUX && tx == 0)
     return ceil_div(L.n[1] + 2, band_rows(L.n[0])) * ceil_div(L.n[2] + 2, kchunk);
   if (kind == PK_FLUX)
@@ -91,12 +96,7 @@ inline int tiles_of(const Layout& L, int kind, int kchunk, int tx = FLUX_TX) {
     return ceil_div(L.n[0] + 1, CELL_BX) * ceil_div(L.n[1] + 1, CELL_BY) *
            ceil_div(L.n[2] + 1, CELL_BZ);
   if (kind == PK_ROWS) return L.n[1] * L.n[2];
-  // ghost slab of axis d, threads mapped linearly over it (FILL_TILE cells
-  // per tile)
-  const int d = kind - PK_FILL0;
-  long long cells = 1;
-  for (int e = 0; e < 3; ++e) cells *= e < d ? L.n[e] + 2 * g + 1 : (e == d ? 2 * g + 1 : L.n[e] + 1);
-  return (int)((cells + FILL_TILE - 1) / FILL_TILE);
+  return (int)((ghost_cells(L) + FILL_TILE - 1) / FILL_TILE);   // PK_FILL
 }
 
 }  // namespace aeth
@@ -126,6 +126,7 @@ struct aeth_ctx {
   unsigned long long* d_floor = nullptr;
   unsigned long long* d_fallback = nullptr;
   double* d_diag = nullptr;      // 8 doubles
+  unsigned* d_arrived = nullptr; // CTAs of a CFL pass that wrote their minimum
   double* d_stage = nullptr;
   double* d_pack = nullptr;           // device copy of the packed state of every
   size_t pack_doubles = 0;            // block (allocated on first use)

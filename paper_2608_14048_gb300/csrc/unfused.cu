@@ -307,7 +307,7 @@ static void stage_unfused(aeth_ctx* c, const BlockPtrs<R>& P, int recon, int src
   ua.beta = beta;
   ua.dt = c->d_dt;
   k_update<R><<<grd, blk, 0, st>>>(L, P.geo, ua, mhd);
-  c->n_launch += 3 + 1 + 3 + (mhd ? 1 : 0) + 1;
+  c->n_launch += 1 + 1 + 3 + (mhd ? 1 : 0) + 1;
 }
 
 template <typename R, bool P64>
