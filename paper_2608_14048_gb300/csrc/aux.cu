@@ -164,7 +164,8 @@ aeth_status build_geometry(aeth_ctx* c) {
 // that runs `slots` tiles at a time takes about the mean load of a slot plus
 // half a tile for the end of the last wave, and at least one tile.  Measured
 // with 32-wide tiles, us per step: 256^3 FP32 3075 (kc 8), 3063 (17), 3079
-// (30), 3150 (64); 128^3 isothermal 458 (8), 459 (17), 475 (32); 64^3 113 (1),
+// (30), 3150 (64); 128^3 isothermal 458 (8), 459 (17), 475 (32); PPM RK3
+// 190 x 131 x 77 1028 (4), 1005 (8), 989 (10), 1016 (14), 1158 (26); 64^3 113 (1),
 // 109 (2 to 6); 32^3 68 (1), 72 (4), 78 (6); FP64 96^3 6960 (4), 7283 (7), 7743
 // (16).  The longest chunk with four tiles an SM, the rule before, took 64, 32
 // and 16 of these.
@@ -174,8 +175,10 @@ static int default_kchunk(const aeth_ctx* c) {
   // FP64: the FP64 pipe of an SM, not a slot, is the unit that runs out, so a
   // whole tile ends late; staging costs next to nothing there
   const bool f64 = c->elem == 8;
-  const double slots = (double)c->num_sms * (f64 ? 2 : (c->flux_tx ? 5 : 2));
-  const double w = f64 ? 0.3 : 1.0, tail = f64 ? 1.0 : 0.5;
+  // PPM and PPM5: one more plane below the chunk, and four tiles an SM
+  const bool ppm = c->cfg.recon == AETH_RECON_PPM || c->cfg.recon == AETH_RECON_PPM5;
+  const double slots = (double)c->num_sms * (f64 ? 2 : (c->flux_tx ? (ppm ? 4 : 5) : 2));
+  const double w = f64 ? 0.3 : (ppm ? 2.0 : 1.0), tail = f64 ? 1.0 : 0.5;
   int best = 1;
   double best_cost = 1e300;
   // the even divisions of the tallest block
