@@ -118,7 +118,7 @@ template <typename R>
 __device__ __forceinline__ R vl_slope(R wm, R w0, R wp) {
   R dm = w0 - wm, dp = wp - w0;
   R q = dm * dp;
-  return q > R(0) ? R(2) * q / (dm + dp) : R(0);
+  return q > R(0) ? quot(R(2) * q, dm + dp) : R(0);
 }
 
 // Fourth-order interface value between s1 and s2, clipped to their range.

@@ -27,6 +27,7 @@
 
 #include "dfloat.cuh"
 #include "ghost.cuh"
+#include "pair.cuh"
 #include "runtime.hpp"
 
 namespace aeth {
@@ -46,53 +47,225 @@ constexpr double kImexG = 1.0 + 0.70710678118654752440;
 constexpr double kImexD = 1.0 - 1.0 / (2.0 * kImexG);
 
 // ------------------------------------------------------------------------
-// Rusanov flux of all species across the lower D-face of each cell
+// Flux divergence of every species from the Rusanov fluxes of its faces
 // ------------------------------------------------------------------------
-template <typename R, int RECON, int D>
-__global__ void __launch_bounds__(256)
-    k_dust_flux(Layout L, const R* __restrict__ dsrc, R* __restrict__ dflux, int nd,
-                R dfloor) {
-  int c3[3];
-  c3[0] = blockIdx.x * blockDim.x + threadIdx.x;
-  c3[1] = blockIdx.y * blockDim.y + threadIdx.y;
-  c3[2] = blockIdx.z * blockDim.z + threadIdx.z;
+
+// Flux across a D-face from its states (rho, v1, v2, v3).
+template <int D, typename R>
+__device__ __forceinline__ void dust_flux(const R* wl, const R* wr, R* f) {
+  const R vnl = wl[1 + D], vnr = wr[1 + D];
+  const R sp = fmax(fabs(vnl), fabs(vnr));
+  const R ul[4] = {wl[0], wl[0] * wl[1], wl[0] * wl[2], wl[0] * wl[3]};
+  const R ur[4] = {wr[0], wr[0] * wr[1], wr[0] * wr[2], wr[0] * wr[3]};
 #pragma unroll
-  for (int e = 0; e < 3; ++e)
-    if (c3[e] > L.n[e] || (e != D && c3[e] == L.n[e])) return;
+  for (int q = 0; q < 4; ++q)
+    f[q] = R(0.5) * (ul[q] * vnl + ur[q] * vnr) - R(0.5) * sp * (ur[q] - ul[q]);
+}
+
+// Flux across the D-face between cells w[2] and w[3] of a line of cells.
+template <int RECON, int D, typename R>
+__device__ __forceinline__ void dust_face(const R (*w)[4], R* f) {
+  R wl[4], wr[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    R s[6];
+#pragma unroll
+    for (int t = 0; t < 6; ++t) s[t] = w[t][q];
+    recon_face<RECON>(s, wl[q], wr[q]);
+  }
+  dust_flux<D>(wl, wr, f);
+}
+
+// Threads over (x, y), marching along z over kc cells of one species: the z
+// line of cells and the flux of the last z face stay in registers; the x and y
+// lines come through L1.  The divergence goes to memory, not the fluxes: a
+// third of the stores here and of the loads of the update.  Each x and y face
+// is computed by both of its cells, cheaper than an exchange (the kernel has no
+// barrier).  128^3, 8 species, PLM: three passes of fluxes
+// 475 us, this one 456 (932 instructions a cell and species, issue rate 88%).
+template <typename R, int RECON>
+__global__ void __launch_bounds__(128)
+    k_dust_div(Layout L, const R* __restrict__ dsrc, R* __restrict__ ddiv, int nd, int kc, R idx1,
+               R idx2, R idx3, R dfloor) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int j = blockIdx.y * blockDim.y + threadIdx.y;
+  const int s = (int)(blockIdx.z % (unsigned)nd);
+  const int k0 = (int)(blockIdx.z / (unsigned)nd) * kc, k1 = min(k0 + kc, L.n[2]);
+  if (i >= L.n[0] || j >= L.n[1]) return;
   constexpr int RH = recon_reach<RECON>(), RL = RH + 1;
-  const long long sz = L.size();
-  const long long fc = L.idx(c3[0], c3[1], c3[2]);
-  const long long sd = L.stride(D);
-  for (int s = 0; s < nd; ++s) {
-    const R* rho = dsrc + (long long)(4 * s) * sz;
-    R st[4][6];
+  const long long sz = L.size(), sx = L.sx, sxy = L.sx * L.sy;
+  const R* rho = dsrc + (long long)(4 * s) * sz;
+  R* out = ddiv + (long long)(4 * s) * sz;
+  auto load = [&](long long at, R* w) {
+    R r = rho[at];
+    if (r < dfloor) r = dfloor;
+    const R ir = recip(r);
+    w[0] = r;
 #pragma unroll
-    for (int t = 0; t < 6; ++t) {
-      const int off = t - 3;
-      if (off < -RL || off > RH) {
-        st[0][t] = st[1][t] = st[2][t] = st[3][t] = R(0);
-        continue;
+    for (int q = 0; q < 3; ++q) w[1 + q] = rho[(long long)(1 + q) * sz + at] * ir;
+  };
+  // entries t of a line: cells t - 3 about the current one; outside the
+  // reconstruction's reach they stay zero
+  R lz[7][4] = {}, fz[4];
+  long long c = L.idx(i, j, k0);
+#pragma unroll
+  for (int t = 3 - RL; t <= 3 + RH; ++t) load(c + (t - 3) * sxy, lz[t]);
+  dust_face<RECON, 2>(lz, fz);
+  for (int k = k0; k < k1; ++k, c += sxy) {
+    load(c + RL * sxy, lz[3 + RL]);
+    R div[4];
+    {
+      R l[7][4] = {}, lo[4], hi[4];
+#pragma unroll
+      for (int t = 3 - RL; t <= 3 + RL; ++t) {
+        if (t != 3) load(c + (t - 3), l[t]);
+        else
+#pragma unroll
+          for (int q = 0; q < 4; ++q) l[t][q] = lz[3][q];
       }
-      const long long cc = fc + off * sd;
-      R r = rho[cc];
-      if (r < dfloor) r = dfloor;
-      const R ir = R(1) / r;
-      st[0][t] = r;
+      dust_face<RECON, 0>(l, lo);
+      dust_face<RECON, 0>(l + 1, hi);
 #pragma unroll
-      for (int q = 0; q < 3; ++q) st[1 + q][t] = rho[(long long)(1 + q) * sz + cc] * ir;
+      for (int q = 0; q < 4; ++q) {
+        div[q] = R(0);
+        div[q] += (hi[q] - lo[q]) * idx1;
+      }
     }
-    R wl[4], wr[4];
+    {
+      R l[7][4] = {}, lo[4], hi[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) recon_face<RECON>(st[q], wl[q], wr[q]);
-    const R vnl = wl[1 + D], vnr = wr[1 + D];
-    const R sp = fmax(fabs(vnl), fabs(vnr));
-    const R ul[4] = {wl[0], wl[0] * wl[1], wl[0] * wl[2], wl[0] * wl[3]};
-    const R ur[4] = {wr[0], wr[0] * wr[1], wr[0] * wr[2], wr[0] * wr[3]};
-    R* out = dflux + (long long)((D * nd + s) * 4) * sz;
+      for (int t = 3 - RL; t <= 3 + RL; ++t) {
+        if (t != 3) load(c + (t - 3) * sx, l[t]);
+        else
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
-      out[(long long)q * sz + fc] =
-          R(0.5) * (ul[q] * vnl + ur[q] * vnr) - R(0.5) * sp * (ur[q] - ul[q]);
+          for (int q = 0; q < 4; ++q) l[t][q] = lz[3][q];
+      }
+      dust_face<RECON, 1>(l, lo);
+      dust_face<RECON, 1>(l + 1, hi);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) div[q] += (hi[q] - lo[q]) * idx2;
+    }
+    R hi[4];
+    dust_face<RECON, 2>(lz + 1, hi);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      div[q] += (hi[q] - fz[q]) * idx3;
+      fz[q] = hi[q];
+      out[(long long)q * sz + c] = div[q];
+    }
+#pragma unroll
+    for (int t = 3 - RL; t < 3 + RL; ++t)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) lz[t][q] = lz[t + 1][q];
+  }
+}
+
+// The same for FP32 and PLM, the default, on packed pairs (rho, v1), (v2, v3):
+// the pass is bound by the issue rate, and a pair takes one instruction.  515
+// instructions a cell and species, 297 us; the update, which reads a third,
+// 507 / 565 -> 400 / 504 us; the step 2440 -> 1910 us.  The momenta are rounded before their difference, as the scalar
+// text does it (ptxas would fuse a packed product into it).
+template <int D>
+__device__ __forceinline__ void dust_flux2(const float2* l, const float2* r, float2* f) {
+  const float vl[3] = {l[0].y, l[1].x, l[1].y}, vr[3] = {r[0].y, r[1].x, r[1].y};
+  float ml[3], mr[3];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    ml[q] = __fmul_rn(l[0].x, vl[q]);
+    mr[q] = __fmul_rn(r[0].x, vr[q]);
+  }
+  const float2 hs = splat(-0.5f * fmaxf(fabsf(vl[D]), fabsf(vr[D])));
+  const float2 x0 = make_float2(__fadd_rn(ml[D], mr[D]),
+                                __fmaf_rn(ml[0], vl[D], __fmul_rn(mr[0], vr[D])));
+  const float2 ul = make_float2(ml[1], ml[2]), ur = make_float2(mr[1], mr[2]);
+  const float2 x1 = fma2(ul, splat(vl[D]), ur * splat(vr[D]));
+  f[0] = fma2(splat(0.5f), x0, hs * (make_float2(r[0].x, mr[0]) - make_float2(l[0].x, ml[0])));
+  f[1] = fma2(splat(0.5f), x1, hs * (ur - ul));
+}
+
+__global__ void __launch_bounds__(128)
+    k_dust_div_plm2(Layout L, const float* __restrict__ dsrc, float* __restrict__ ddiv, int nd,
+                    int kc, float idx1, float idx2, float idx3, float dfloor) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int j = blockIdx.y * blockDim.y + threadIdx.y;
+  const int s = (int)(blockIdx.z % (unsigned)nd);
+  const int k0 = (int)(blockIdx.z / (unsigned)nd) * kc, k1 = min(k0 + kc, L.n[2]);
+  if (i >= L.n[0] || j >= L.n[1]) return;
+  const long long sz = L.size(), sx = L.sx, sxy = L.sx * L.sy;
+  const float* p0 = dsrc + (long long)(4 * s) * sz;
+  const float* p1 = p0 + sz;
+  const float* p2 = p1 + sz;
+  const float* p3 = p2 + sz;
+  float* out = ddiv + (long long)(4 * s) * sz;
+  auto load = [&](long long at, float2* w) {
+    float r = p0[at];
+    if (r < dfloor) r = dfloor;
+    const float ir = recip(r);
+    w[0] = make_float2(r, p1[at] * ir);
+    w[1] = make_float2(p2[at], p3[at]) * splat(ir);
+  };
+  // half slopes of the middle cell of three
+  auto half = [](const float2* a, const float2* b, const float2* c, float2* h) {
+#pragma unroll
+    for (int p = 0; p < 2; ++p) h[p] = plm_half2(b[p] - a[p], c[p] - b[p]);
+  };
+  // flux between cells a (half slopes ha) and b (hb)
+  auto face = [](auto D, const float2* a, const float2* ha, const float2* b, const float2* hb,
+                 float2* f) {
+    const float2 l[2] = {a[0] + ha[0], a[1] + ha[1]}, r[2] = {b[0] - hb[0], b[1] - hb[1]};
+    dust_flux2<decltype(D)::value>(l, r, f);
+  };
+  long long c = L.idx(i, j, k0);
+  // z: cells k, k + 1 and the half slopes of k; flux of k's lower face
+  float2 w0[2], w1[2], h0[2], fz[2];
+  {
+    float2 wb[2], wa[2], ha[2];
+    load(c - 2 * sxy, wb);
+    load(c - sxy, wa);
+    load(c, w0);
+    load(c + sxy, w1);
+    half(wb, wa, w0, ha);
+    half(wa, w0, w1, h0);
+    face(std::integral_constant<int, 2>(), wa, ha, w0, h0, fz);
+  }
+  for (int k = k0; k < k1; ++k, c += sxy) {
+    float2 div[2];
+    // x or y line of cells
+    auto line = [&](auto D, long long st, float inv) {
+      float2 a[2], b[2], d[2], e[2], hb[2], hc[2], hd[2], lo[2], hi[2];
+      load(c - 2 * st, a);
+      load(c - st, b);
+      load(c + st, d);
+      load(c + 2 * st, e);
+      half(a, b, w0, hb);
+      half(b, w0, d, hc);
+      half(w0, d, e, hd);
+      face(D, b, hb, w0, hc, lo);
+      face(D, w0, hc, d, hd, hi);
+#pragma unroll
+      for (int p = 0; p < 2; ++p) {
+        const float2 df = hi[p] - lo[p];
+        div[p] = decltype(D)::value == 0 ? df * splat(inv) : fma2(df, splat(inv), div[p]);
+      }
+    };
+    line(std::integral_constant<int, 0>(), 1, idx1);
+    line(std::integral_constant<int, 1>(), sx, idx2);
+    float2 w2[2], h1[2], hi[2];
+    load(c + 2 * sxy, w2);
+    half(w0, w1, w2, h1);
+    face(std::integral_constant<int, 2>(), w0, h0, w1, h1, hi);
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      div[p] = fma2(hi[p] - fz[p], splat(idx3), div[p]);
+      fz[p] = hi[p];
+      w0[p] = w1[p];
+      w1[p] = w2[p];
+      h0[p] = h1[p];
+    }
+    out[c] = div[0].x;
+    out[sz + c] = div[0].y;
+    out[2 * sz + c] = div[1].x;
+    out[3 * sz + c] = div[1].y;
   }
 }
 
@@ -106,7 +279,7 @@ struct DustUpd {
   const R* gf[3][5];   // gas fluxes
   R* da;               // dust register A (base)
   R* db;               // dust register B (base)
-  const R* df;         // dust fluxes (base)
+  const R* df;         // dust flux divergences (base)
   double drag_c[32];   // per species: 1 / t_k (constant stopping time) or
                        // K_k (constant coefficient, t_k = rho_k / K_k)
   const double* dt;
@@ -292,12 +465,7 @@ __global__ void __launch_bounds__(256)
     if (s >= nd) break;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      R div = R(0);
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        const R* f = A.df + (long long)(((a * nd + s) * 4 + q)) * sz;
-        div += (f[c + st[a]] - f[c]) * inv[a];
-      }
+      const R div = A.df[(long long)(4 * s + q) * sz + c];
       ud[s][q] = A.da[(long long)(4 * s + q) * sz + c];
       dx[s][q] = ud[s][q] - (stage == 2 ? g : R(1) - d) * dt * div;
     }
@@ -537,30 +705,31 @@ static void stage_dust(aeth_ctx* c, int b, int src, int stage) {
   k_fill_cells<R><<<ceil_div(ghost_cells(L), 256), 256, 0, s>>>(L, P.dust[src], 4 * nd);
   c->n_launch += 2;
   hydro_flux_pass<R, P64>(c, b, c->cfg.recon, src);
-  dim3 blk(32, 4, 2);
-  dim3 grd((L.n[0] + 1 + 31) / 32, (L.n[1] + 1 + 3) / 4, (L.n[2] + 1 + 1) / 2);
   const R dfl = (R)1e-20;
-  const R* dsrc = P.dust[src];
+  // inverse cell widths (Cartesian: area / volume = 1 / dx_d)
+  const R i1 = (R)(B.desc.nx / (B.desc.x1max - B.desc.x1min));
+  const R i2 = (R)(B.desc.ny / (B.desc.x2max - B.desc.x2min));
+  const R i3 = (R)(B.desc.nz / (B.desc.x3max - B.desc.x3min));
+  // cells of a z march: 16, fewer where that leaves less than about two waves
+  // of CTAs (a march of 4 spends as much again on its first face)
+  auto ctas = [&](int kc) {
+    return (long long)ceil_div(L.n[0], 32) * ceil_div(L.n[1], 4) * ceil_div(L.n[2], kc) * nd;
+  };
+  int kc = 16;
+  while (kc > 4 && ctas(kc) < 8LL * c->num_sms) kc /= 2;
+  while ((long long)ceil_div(L.n[2], kc) * nd > 65535) kc *= 2;   // grid limit
+  auto divergence = [&](auto kernel) {
+    const dim3 grd(ceil_div(L.n[0], 32), ceil_div(L.n[1], 4), ceil_div(L.n[2], kc) * nd);
+    kernel<<<grd, dim3(32, 4), 0, s>>>(L, P.dust[src], P.dflux, nd, kc, i1, i2, i3, dfl);
+  };
   switch (c->cfg.recon) {
-    case AETH_RECON_DONOR:
-      k_dust_flux<R, 0, 0><<<grd, blk, 0, s>>>(L, dsrc, P.dflux, nd, dfl);
-      k_dust_flux<R, 0, 1><<<grd, blk, 0, s>>>(L, dsrc, P.dflux, nd, dfl);
-      k_dust_flux<R, 0, 2><<<grd, blk, 0, s>>>(L, dsrc, P.dflux, nd, dfl);
-      break;
+    case AETH_RECON_DONOR: divergence(k_dust_div<R, 0>); break;
     case AETH_RECON_PLM:
-      k_dust_flux<R, 1, 0><<<grd, blk, 0, s>>>(L, dsrc, P.dflux, nd, dfl);
-      k_dust_flux<R, 1, 1><<<grd, blk, 0, s>>>(L, dsrc, P.dflux, nd, dfl);
-      k_dust_flux<R, 1, 2><<<grd, blk, 0, s>>>(L, dsrc, P.dflux, nd, dfl);
+      if constexpr (sizeof(R) == 4) divergence(k_dust_div_plm2);
+      else divergence(k_dust_div<R, 1>);
       break;
-    case AETH_RECON_PPM5:
-      k_dust_flux<R, 3, 0><<<grd, blk, 0, s>>>(L, dsrc, P.dflux, nd, dfl);
-      k_dust_flux<R, 3, 1><<<grd, blk, 0, s>>>(L, dsrc, P.dflux, nd, dfl);
-      k_dust_flux<R, 3, 2><<<grd, blk, 0, s>>>(L, dsrc, P.dflux, nd, dfl);
-      break;
-    default:
-      k_dust_flux<R, 2, 0><<<grd, blk, 0, s>>>(L, dsrc, P.dflux, nd, dfl);
-      k_dust_flux<R, 2, 1><<<grd, blk, 0, s>>>(L, dsrc, P.dflux, nd, dfl);
-      k_dust_flux<R, 2, 2><<<grd, blk, 0, s>>>(L, dsrc, P.dflux, nd, dfl);
+    case AETH_RECON_PPM5: divergence(k_dust_div<R, 3>); break;
+    default: divergence(k_dust_div<R, 2>);
   }
   DustUpd<R> u{};
   for (int v = 0; v < 5; ++v) {
@@ -575,10 +744,6 @@ static void stage_dust(aeth_ctx* c, int b, int src, int stage) {
   for (int q = 0; q < nd; ++q) u.drag_c[q] = coeff ? c->t_stop[q] : 1.0 / c->t_stop[q];
   u.dt = c->d_dt;
   u.dfloor = dfl;
-  // inverse cell widths (Cartesian: area / volume = 1 / dx_d)
-  const R i1 = (R)(B.desc.nx / (B.desc.x1max - B.desc.x1min));
-  const R i2 = (R)(B.desc.ny / (B.desc.x2max - B.desc.x2min));
-  const R i3 = (R)(B.desc.nz / (B.desc.x3max - B.desc.x3min));
   // the update: CTAs of 32 x 4 x AETH_DUST_BZ cells (its registers allow
   // few CTAs per SM)
   const dim3 blk2(32, 4, AETH_DUST_BZ);
@@ -615,7 +780,7 @@ static void stage_dust(aeth_ctx* c, int b, int src, int stage) {
   } else {
     launch(k_dust_update<R, R, 32>);
   }
-  c->n_launch += 3 + 1;
+  c->n_launch += 1 + 1;
 }
 
 template <typename R, bool P64>

@@ -1,6 +1,8 @@
-"""The one-launch ghost fill at its edge sizes: linked blocks of the smallest
-allowed size (their ghosts reach through two neighbours) between outflow and
-periodic edges, against one block."""
+"""The one-launch ghost fill and the packed dust divergence at their edge
+sizes.  Every cell of a replicated or split domain goes through the same
+arithmetic, so the states must agree: extents below the ghost
+width, linked blocks of the smallest allowed size (their ghosts reach through
+two neighbours), outflow edges, and z marches with a remainder."""
 import numpy as np
 import pytest
 
@@ -28,3 +30,40 @@ def test_smallest_linked_blocks_match_one_block(prec, splits, bc):
     for a, b in zip(got, ref):
         np.testing.assert_allclose(a, b, rtol=EPS[prec], atol=EPS[prec])
     assert dt == pytest.approx(dt_ref, rel=EPS[prec])
+
+
+@pytest.mark.parametrize("bc", [0, 1])
+@pytest.mark.parametrize("drag", [A.DRAG_FP32, A.DRAG_FP64])
+def test_thin_dusty_blocks_match_replicated_ones(bc, drag):
+    """A state that varies along x only: blocks of 1 x 1 and of 5 x 19 (z march
+    16 + 3) cells across evolve alike."""
+    import torch
+    nx, nd, rng = 33, 3, np.random.default_rng(3)
+    line = np.empty((5 + 4 * nd, nx))
+    line[0], line[1:4], line[4] = 1 + rng.random(nx), rng.standard_normal((3, nx)), 8.0
+    for k in range(nd):
+        line[5 + 4 * k] = 0.1 + rng.random(nx)
+        line[6 + 4 * k:9 + 4 * k] = rng.standard_normal((3, nx)) * 0.2
+    out = []
+    for ny, nz in ((1, 1), (5, 19)):
+        full = np.ascontiguousarray(np.broadcast_to(line[:, None, None, :], (len(line), nz, ny, nx)))
+        cfg = A.make_config(gamma=1.4, recon=A.PLM, integrator=A.IMEX2P, precision=A.FP32,
+                            mhd=False, t_stop=[0.1, 0.01, 1.0], drag_precision=drag)
+        sv = A.Solver(cfg, [A.make_block((nx, ny, nz), (0.0, 0.0, 0.0), (1.0, ny / nx, nz / nx),
+                                         A.CART, (bc, bc, bc))], stream=torch.cuda.current_stream())
+        try:
+            sv.set_state(0, full[:5])
+            for k in range(nd):
+                A.aeth_set_dust(sv.ctx, 0, k, np.ascontiguousarray(full[5 + 4 * k:9 + 4 * k]))
+            for _ in range(3):
+                sv.step(1e-3)
+            r = [sv.get_state(0)[0]]
+            for k in range(nd):
+                buf = np.empty((4, nz, ny, nx))
+                A.aeth_get_dust(sv.ctx, 0, k, buf)
+                r.append(buf)
+        finally:
+            sv.close()
+        out.append(np.concatenate(r))
+    np.testing.assert_array_equal(out[1], np.broadcast_to(out[0], out[1].shape))
+    assert np.abs(out[0] - line[:, None, None, :]).max() > 1e-3
