@@ -79,16 +79,17 @@ __host__ __device__ constexpr int flux_ring() { return recon_reach<RECON>() + 2;
 constexpr bool iso_solver(int solver) { return solver == 3 || solver == 4; }
 
 // Riemann solver family SOLVER (numbering of k_flux3 below) on one face: on
-// packed pairs in FP32 (HLLD, LHLLD, isothermal HLLD), else the scalar solvers;
+// packed pairs in FP32 (all but the isothermal HLLE), else the scalar solvers;
 // a gas without field takes either without its terms.  SPLIT: see riemann2.cuh;
 // set for the z faces of donor-cell states, whose rounding it fixes.
 template <int SOLVER, bool MHD, bool SPLIT, typename R>
 __device__ __forceinline__ void solve_face(R g, R igm1, const R* wl, const R* wr, R bn, R* fx) {
-  if constexpr (sizeof(R) == 4 && SOLVER != 2 && SOLVER != 4) {
+  if constexpr (sizeof(R) == 4 && SOLVER != 4) {
     float2 W[7];
 #pragma unroll
     for (int v = 0; v < 7; ++v) W[v] = make_float2(wl[v], wr[v]);
-    if constexpr (SOLVER == 3) hlld_iso2<MHD, SPLIT>(g * g, W, bn, fx);
+    if constexpr (SOLVER == 2) hlle2<MHD>(g, igm1, W, bn, fx);
+    else if constexpr (SOLVER == 3) hlld_iso2<MHD, SPLIT>(g * g, W, bn, fx);
     else hlld2<SOLVER == 5, MHD, SPLIT>(g, igm1, W, bn, fx);
   } else {
     if constexpr (SOLVER == 2) hlle<MHD>(g, wl, wr, bn, fx);
