@@ -219,7 +219,7 @@ def peaks():
     return 6800.0, "fallback"
 
 
-KERNEL_SOURCES = ("flux3.cuh", "common.cuh", "stage.cuh")
+KERNEL_SOURCES = ("flux3.cuh", "common.cuh", "stage.cuh", "pair.cuh", "riemann2.cuh")
 
 
 def nvtx_push(name):

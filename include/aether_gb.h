@@ -434,8 +434,8 @@ aeth_status aeth_profile_read(aeth_ctx* ctx, double* total_ms,
  * narrower than a 2-D tile busy (every block at most 64 cells wide).  16 and 0 are built for FP32
  * and FP32_P64 / FP32_SEL64 contexts with a classical solver, no dual
  * energy, fused path (AETH_ERR_UNSUPPORTED otherwise); kchunk in 1 .. 1024 (the
- * default is the largest of 64, 32, 16, 8, 4 that gives every SM four
- * tiles).  Each face is solved once, by the same code, whatever the shape:
+ * default divides the tallest block evenly, as the load of the SMs makes it
+ * cheapest).  Each face is solved once, by the same code, whatever the shape:
  * the 2-D shapes give identical states, band tiles states within a few
  * FP32 ulps of them (the compiler contracts some multiply-adds of that
  * kernel differently).  aeth_set_flux_tile rebuilds the launch tables

@@ -1,7 +1,7 @@
 // Multifluid dust (Sec. 2.2, Eqs. 6-7) with the IMEX2P integrator (Sec. 2.6).
 //
 // Per stage: ghost fill; the fused hydro-gas flux pass (HLLD at B = 0);
-// one pressureless Rusanov flux pass per direction for all species; then one
+// one pass for the divergence of every species' pressureless Rusanov fluxes; then one
 // fused kernel that forms the explicit stage combination and solves the
 // implicit drag of every cell in closed form (arrowhead system, O(N) per
 // velocity component) in FP64 by default (aeth_config.drag_precision),
@@ -12,9 +12,10 @@
 // conversions a cell made the update 68% of the step, so FP32 transport solves
 // in FP32 pairs (dfloat.cuh, about 48 bits: the same FP32 results but for rare
 // last bits; error against FP64 of 10 steps unchanged, 1.4e-7).  128^3, 8
-// species: the update 1751 -> 458 / 565 us a launch (1.6 and 2.2 GB: now bound
-// by memory latency at 16 warps an SM), the step 5169 -> 2504 us; 61 x 100 x 37,
-// 3 species, per-species precision: 395 -> 273 us a step.  The FP64 solve stays
+// species: the update 1751 -> 458 / 565 us a launch (now 400 / 504 on the
+// divergence, 1.0 and 1.4 GB: bound by memory latency at 16 warps an SM and the
+// pairs' serial sums), the step 5169 -> 2504 us; 61 x 100 x 37, 3 species,
+// per-species precision: 395 -> 273 us a step.  The FP64 solve stays
 // for FP64 transport, the constant-coefficient law, and cells or constants
 // outside the pairs' range.
 //

@@ -3,9 +3,8 @@
 // Every pass is ONE launch over all mesh blocks of the context: a device
 // table holds each block's layout, geometry and array pointers, and each
 // pass kind has a prefix sum of tiles per block, so a CTA finds its block
-// by binary search.  The flux pass is persistent (grid-stride over tiles,
-// grid sized to the SM count); uneven block sizes only change the number
-// of tiles per block.
+// by binary search or from a tile map; uneven block sizes only change the
+// number of tiles per block.
 //
 //  1. k_flux3 (flux3.cuh): conserved->primitive, reconstruction and the
 //     Riemann solver for all three face directions of every cell in one
