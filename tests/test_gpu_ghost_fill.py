@@ -33,8 +33,9 @@ def test_smallest_linked_blocks_match_one_block(prec, splits, bc):
 
 
 @pytest.mark.parametrize("bc", [0, 1])
-@pytest.mark.parametrize("drag", [A.DRAG_FP32, A.DRAG_FP64])
-def test_thin_dusty_blocks_match_replicated_ones(bc, drag):
+@pytest.mark.parametrize("recon,drag", [(A.PLM, A.DRAG_FP32), (A.PLM, A.DRAG_FP64), (A.DONOR, A.DRAG_FP64),
+                                        (A.PPM, A.DRAG_FP64), (A.PPM5, A.DRAG_SEL64)])
+def test_thin_dusty_blocks_match_replicated_ones(bc, recon, drag):
     """A state that varies along x only: blocks of 1 x 1 and of 5 x 19 (z march
     16 + 3) cells across evolve alike."""
     import torch
@@ -47,7 +48,7 @@ def test_thin_dusty_blocks_match_replicated_ones(bc, drag):
     out = []
     for ny, nz in ((1, 1), (5, 19)):
         full = np.ascontiguousarray(np.broadcast_to(line[:, None, None, :], (len(line), nz, ny, nx)))
-        cfg = A.make_config(gamma=1.4, recon=A.PLM, integrator=A.IMEX2P, precision=A.FP32,
+        cfg = A.make_config(gamma=1.4, recon=recon, integrator=A.IMEX2P, precision=A.FP32,
                             mhd=False, t_stop=[0.1, 0.01, 1.0], drag_precision=drag)
         sv = A.Solver(cfg, [A.make_block((nx, ny, nz), (0.0, 0.0, 0.0), (1.0, ny / nx, nz / nx),
                                          A.CART, (bc, bc, bc))], stream=torch.cuda.current_stream())
