@@ -390,8 +390,14 @@ __device__ __noinline__ void drag_far(const float* gx, const float (*dx)[4], int
 // COEFF: the constant-coefficient drag law (drag_c = K_k, a_k = h K_k /
 // rho_k per cell).  iso: isothermal gas, whose energy slot takes no drag
 // heating.
+// Bounds: five CTAs of 128 threads an SM for the solve in pairs of up to 8 species
+// (102 registers): 128^3, 8 species, step 1909 -> 1897 us against the compiler's own
+// 128 registers; 61 x 100 x 37, 3 species 210 -> 205.  The others keep what they need.
+template <typename DT, int NDMAX>
+constexpr bool upd_five = std::is_same_v<DT, dfloat> && NDMAX <= 8;
 template <typename R, typename DT, int NDMAX, bool SEL = false, bool COEFF = false>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(upd_five<DT, NDMAX> ? 128 * AETH_DUST_BZ : 256,
+                                  upd_five<DT, NDMAX> ? 5 / AETH_DUST_BZ : 0)
     k_dust_update(Layout L, R idx1, R idx2, R idx3, DustUpd<R> A, int nd, int stage,
                   unsigned long long* floor_hits, float sel_ratio, int iso) {
   // per-species drag constants of this stage, the same for every cell:
