@@ -169,16 +169,28 @@ aeth_status build_geometry(aeth_ctx* c) {
 // 109 (2 to 6); 32^3 68 (1), 72 (4), 78 (6); FP64 96^3 6960 (4), 7283 (7), 7743
 // (16).  The longest chunk with four tiles an SM, the rule before, took 64, 32
 // and 16 of these.
+// FP32_P64 recovers every staged cell's pressure in FP64, so the FP64 pipe of
+// the SMs bounds the pass, through the warm-up planes too (w 2), and tiles go
+// in waves: a wave costs as many tiles as an SM holds, and the last one never
+// less than four, whose warps the pipe needs to stay busy.  us per step, by
+// this rule and by the one above: PLM 64^3 191 (kc 6), 229 (3); 150 x 20 x 60 158 (4),
+// 199 (2); hydro 34 x 124 x 42 129 (5), 163 (3); PPM 80^3 382 (10), 445 (6).  Over 60
+// combinations of sizes, reconstructions and closures it is within 9% of the best
+// chunk, the one above up to 28% off.
 static int default_kchunk(const aeth_ctx* c) {
   int nzmax = 1;
   for (const auto& B : c->blocks) nzmax = std::max(nzmax, B.L.n[2]);
   // FP64: the FP64 pipe of an SM, not a slot, is the unit that runs out, so a
-  // whole tile ends late; staging costs next to nothing there
+  // whole tile ends late; staging costs next to nothing there.  Tiles that fit
+  // one wave run 1.35 times a tile's time: 17 x 160 x 24 hydro PLM 623 us (kc 4, 287
+  // tiles) against 688 (kc 1)
   const bool f64 = c->elem == 8;
   // PPM and PPM5: one more plane below the chunk, and four tiles an SM
   const bool ppm = c->cfg.recon == AETH_RECON_PPM || c->cfg.recon == AETH_RECON_PPM5;
-  const double slots = (double)c->num_sms * (f64 ? 2 : (c->flux_tx ? (ppm ? 4 : 5) : 2));
-  const double w = f64 ? 0.3 : (ppm ? 2.0 : 1.0), tail = f64 ? 1.0 : 0.5;
+  const bool p64 = c->cfg.precision == AETH_FP32_P64 && !is_iso(c);
+  const int per_sm = f64 ? 2 : (c->flux_tx ? (ppm ? 4 : 5) : 2);
+  const double slots = (double)c->num_sms * per_sm;
+  const double w = f64 ? 0.3 : (ppm || p64 ? 2.0 : 1.0), tail = f64 ? 1.0 : 0.5;
   int best = 1;
   double best_cost = 1e300;
   // the even divisions of the tallest block
@@ -186,11 +198,20 @@ static int default_kchunk(const aeth_ctx* c) {
     const int kc = ceil_div(nzmax + 2, parts);
     if (kc > 64 || ceil_div(nzmax + 2, kc) != parts) continue;
     double planes = 0;
+    long long tiles = 0;
     for (const auto& B : c->blocks) {
       const double chunks = ceil_div(B.L.n[2] + 2, kc);
-      planes += tiles_of(B.L, PK_FLUX, kc, c->flux_tx) / chunks * (B.L.n[2] + 2 + w * chunks);
+      const int t = tiles_of(B.L, PK_FLUX, kc, c->flux_tx);
+      tiles += t;
+      planes += t / chunks * (B.L.n[2] + 2 + w * chunks);
     }
-    const double cost = std::max(kc + w, planes / slots + tail * (kc + w));
+    double cost = std::max(kc + w, planes / slots + tail * (kc + w));
+    if (f64 && tiles <= slots) cost = 1.35 * (kc + w);
+    if (p64) {
+      const long long wave = (long long)c->num_sms * per_sm, rest = tiles % wave;
+      const int last = rest ? std::max(ceil_div(rest, c->num_sms), std::min(4, per_sm)) : 0;
+      cost = ((double)(tiles / wave) * per_sm + last) * (kc + w);
+    }
     if (cost < best_cost) {
       best_cost = cost;
       best = kc;
