@@ -248,7 +248,8 @@ aeth_status aeth_plan(aeth_ctx* c, size_t* bytes) {
         off += align256((size_t)4 * c->cfg.n_dust * sz * c->elem);
       }
       B.off_dflux = off;
-      off += align256((size_t)4 * c->cfg.n_dust * sz * c->elem);
+      // FP32 keeps the divergences, FP64 the fluxes of three directions
+      off += align256((size_t)(c->elem == 8 ? 12 : 4) * c->cfg.n_dust * sz * c->elem);
     }
     if (c->cfg.riemann == AETH_RIEMANN_MLP) {
       B.off_fstate = off;

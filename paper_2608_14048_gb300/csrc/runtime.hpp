@@ -23,7 +23,8 @@ struct BlockPtrs {
   R* e[3][2];          // face EMFs per direction: components t1, t2
   R* edge[3];          // corner EMFs by component
   R* dust[2];          // dust registers: [species][4] arrays each (IMEX2P)
-  R* dflux;            // dust flux divergences: [species][4] arrays
+  R* dflux;            // dust flux divergences: [species][4] arrays; FP64: fluxes,
+                       // [direction][species][4]
   R* fstate;           // learned flux: face states [direction][wl 7, wr 7, bn]
   const BlockPtrs* tab; // device table of every block of the context (linked
                         // blocks reach their neighbours through it)
@@ -41,7 +42,7 @@ struct BlockInfo {
   size_t off_scratch;     // unfused scratch (w, f, e, edge)
   size_t off_geo;         // geometry tables (R)
   size_t off_dust[2];     // dust registers (n_dust * 4 arrays each)
-  size_t off_dflux;       // dust flux divergences [n_dust][4] arrays
+  size_t off_dflux;       // dust flux divergences [n_dust][4] (FP64: fluxes [3][n_dust][4]) arrays
   size_t off_fstate;      // learned flux: face states [3][15] arrays
   size_t off_ent[2];      // dual energy: entropy array of each register
   size_t geo_len;         // number of R entries in the geometry tables
