@@ -717,7 +717,7 @@ __global__ void __launch_bounds__(upd_five<DT, NDMAX> ? 128 * AETH_DUST_BZ : 256
       for (int q = 0; q < 4; ++q) A.da[(long long)(4 * s + q) * sz + c] = dy[s][q];
     }
   }
-  if (hits) atomicAdd(floor_hits, (unsigned long long)hits);
+  add_hits(floor_hits, hits);
 }
 
 // Ghost fill of narr cell-centred arrays at base + a * sz.

@@ -686,7 +686,7 @@ __global__ void __launch_bounds__(flux_threads(TXT), (flux_minb<R, RECON>(TXT)))
       }
     }
   }
-  if (hits) atomicAdd(floor_hits, (unsigned long long)hits);
+  add_hits(floor_hits, hits);
 }
 
 // ------------------------------------------------------------------------

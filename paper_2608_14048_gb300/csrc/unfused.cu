@@ -58,7 +58,7 @@ __global__ void k_prim(Layout L, ConstArr8<R> u, Arr8<R> w, int mhd, double gamm
   if (cs2 <= 0.0 && pr < p_floor) { pr = p_floor; ++hits; }
   w.p[0][c] = rho; w.p[1][c] = v1; w.p[2][c] = v2; w.p[3][c] = v3;
   w.p[4][c] = pr; w.p[5][c] = b1; w.p[6][c] = b2; w.p[7][c] = b3;
-  if (hits) atomicAdd(floor_hits, (unsigned long long)hits);
+  add_hits(floor_hits, hits);
 }
 
 // ------------------------------------------------------------------------
