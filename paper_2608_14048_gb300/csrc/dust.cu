@@ -370,7 +370,7 @@ __device__ __forceinline__ bool drag_pairs(const float* gx, const float (*dx)[4]
       } else {
         const float m1 = (m0 + rk * fak[s] * vgf) * fia[s];
         dy[s][1 + q] = m1;
-        dke2 = dke2 + (m1 - m0) * (m1 + m0) * (1.0f / rk);
+        dke2 = dke2 + (m1 - m0) * (m1 + m0) * (rk > 0.0f ? 1.0f / rk : 0.0f);
       }
     }
   }
@@ -380,40 +380,99 @@ __device__ __forceinline__ bool drag_pairs(const float* gx, const float (*dx)[4]
   return fabsf(dke2.h) < 1e37f;
 }
 
-// The same in FP64 for the cells the pairs do not take: species with no
-// density (rho_k <= 0) keep their kinetic energy out of the balance.
+// The same in FP64 for the cells the pairs do not take (species with no density,
+// rho_k <= 0, keep their kinetic energy out of the balance).  Such a cell is not
+// rare everywhere: a species at its floor over part of the box, gas in units with
+// densities below 1e-10, an implicit weight beyond the pairs' range.  Bound by the
+// FP64 pipe, so up to 8 species share one division (as k_dust_update's solve in
+// FP64 does), each density is inverted once for the three components, and a
+// species' heat is scaled once.  One uncoupled species, so every cell here: 61 x 100 x
+// 37, 3 species 351 -> 245 us a step (solving in FP64 only: 372), 48^3, 12 species 762 ->
+// 582 (668), 96^3, 4 species 1385 -> 925 (1390).
 template <int NDMAX, bool SEL>
 __device__ __noinline__ void drag_far(const float* gx, const float (*dx)[4], int nd,
                                       const double* ak, const double* ia, const double* wk,
                                       const float* fak, const float* fia, const float* fwk,
                                       unsigned wide, int iso, float* gy, float (*dy)[4]) {
+  constexpr int UN = NDMAX <= 8 ? NDMAX : 1;   // unrolled: the arrays stay in registers
+  auto in64 = [&](int s) { return !SEL || ((wide >> s) & 1u); };
   const double rg = gx[0];
-  double den = rg;
-  for (int s = 0; s < nd; ++s)
-    den += !SEL || ((wide >> s) & 1u) ? (double)dx[s][0] * wk[s] : (double)(dx[s][0] * fwk[s]);
-  const double inv_den = 1.0 / den;
-  double dke2 = 0.0;
+  double den = rg, rk[NDMAX], ir[NDMAX];   // rho_k, 1 / rho_k
+#pragma unroll UN
+  for (int s = 0; s < NDMAX; ++s) {
+    if (s >= nd) break;
+    rk[s] = dx[s][0];
+    den += in64(s) ? rk[s] * wk[s] : (double)(dx[s][0] * fwk[s]);
+  }
+  double inv_den;
+  if constexpr (!SEL && NDMAX <= 8) {
+    // simultaneous inversion: prefix products of the densities (a non-positive
+    // one enters as 1), one division, back-substitution
+    double acc = 1.0;
+#pragma unroll
+    for (int s = 0; s < NDMAX; ++s) {
+      if (s >= nd) break;
+      ir[s] = acc;
+      acc *= dx[s][0] > 0.0f ? rk[s] : 1.0;
+    }
+    const double q = 1.0 / (acc * den);
+    inv_den = q * acc;
+    double ip = q * den;   // 1 / (x_0 ... x_s)
+#pragma unroll
+    for (int s = NDMAX - 1; s >= 0; --s) {
+      if (s >= nd) continue;
+      const bool on = dx[s][0] > 0.0f;
+      ir[s] = on ? ip * ir[s] : 0.0;
+      ip *= on ? rk[s] : 1.0;
+    }
+  } else {
+    inv_den = 1.0 / den;
+#pragma unroll UN
+    for (int s = 0; s < NDMAX; ++s) {
+      if (s >= nd) break;
+      ir[s] = in64(s) && dx[s][0] > 0.0f ? 1.0 / rk[s] : 0.0;
+    }
+  }
+  // twice the change of the dust kinetic energy: the FP32 species' as they come, the
+  // others' times rho_k, summed over the components before the product with 1 / rho_k
+  double dke2 = 0.0, dm2[NDMAX];
+#pragma unroll UN
+  for (int s = 0; s < NDMAX; ++s) {
+    if (s >= nd) break;
+    rk[s] *= ak[s];   // rho_k a_k from here on
+    dm2[s] = 0.0;
+  }
+#pragma unroll 1
   for (int q = 0; q < 3; ++q) {
-    double num = gx[1 + q];
-    for (int s = 0; s < nd; ++s)
-      num += !SEL || ((wide >> s) & 1u) ? wk[s] * (double)dx[s][1 + q]
-                                        : (double)(fwk[s] * dx[s][1 + q]);
+    double num = gx[1 + q], m0[NDMAX];
+#pragma unroll UN
+    for (int s = 0; s < NDMAX; ++s) {
+      if (s >= nd) break;
+      m0[s] = dx[s][1 + q];
+      num += in64(s) ? wk[s] * m0[s] : (double)(fwk[s] * dx[s][1 + q]);
+    }
     const double vg = num * inv_den;
     gy[1 + q] = (float)(rg * vg);
     const float vgf = (float)vg;
-    for (int s = 0; s < nd; ++s) {
-      if (!SEL || ((wide >> s) & 1u)) {
-        const double rk = dx[s][0], m0 = dx[s][1 + q];
-        const double m1 = (m0 + rk * ak[s] * vg) * ia[s];
+#pragma unroll UN
+    for (int s = 0; s < NDMAX; ++s) {
+      if (s >= nd) break;
+      if (in64(s)) {
+        const double m1 = (m0[s] + rk[s] * vg) * ia[s];
         dy[s][1 + q] = (float)m1;
-        if (rk > 0.0) dke2 += (m1 - m0) * (m1 + m0) / rk;
+        dm2[s] += (m1 - m0[s]) * (m1 + m0[s]);
       } else {
-        const float rk = dx[s][0], m0 = dx[s][1 + q];
-        const float m1 = (m0 + rk * fak[s] * vgf) * fia[s];
+        const float r = dx[s][0], mf = dx[s][1 + q];
+        const float m1 = (mf + r * fak[s] * vgf) * fia[s];
         dy[s][1 + q] = m1;
-        if (rk > 0.0f) dke2 += (double)((m1 - m0) * (m1 + m0) * (1.0f / rk));
+        if (r > 0.0f) dke2 += (double)((m1 - mf) * (m1 + mf) * (1.0f / r));
       }
     }
+  }
+#pragma unroll UN
+  for (int s = 0; s < NDMAX; ++s) {
+    if (s >= nd) break;
+    dke2 += dm2[s] * ir[s];
   }
   gy[0] = gx[0];
   gy[4] = iso ? gx[4] : (float)((double)gx[4] - 0.5 * dke2);
@@ -464,7 +523,9 @@ __global__ void __launch_bounds__(upd_five<DT, NDMAX> ? 128 * AETH_DUST_BZ : 256
         s_ak[tid] = dfloat::of(a);
         s_ia[tid] = dfloat::of(ia);
         s_wk[tid] = dfloat::of(a * ia);
-        if (!(a > kPairLo && a < kPairHi)) s_far = 1;
+        // a constant of a species that the pairs solve (an uncoupled FP32 species sent
+        // every cell to FP64: 64^3, 4 species 392 us a step, 200 now)
+        if ((!SEL || a > (CT)sel_ratio) && !(a > kPairLo && a < kPairHi)) s_far = 1;
       } else {
         s_ak[tid] = a;
         s_ia[tid] = ia;
@@ -544,7 +605,9 @@ __global__ void __launch_bounds__(upd_five<DT, NDMAX> ? 128 * AETH_DUST_BZ : 256
     for (int s = 0; s < NDMAX; ++s) {
       if (s >= nd) break;
       dy[s][0] = dx[s][0];
-      far = far || !(dx[s][0] > (R)kPairLo && dx[s][0] < (R)kPairHi);
+      // an FP32 species has no lower bound
+      const bool low = !SEL || ((s_wide >> s) & 1u) ? !(dx[s][0] > (R)kPairLo) : false;
+      far = far || low || !(fabsf(dx[s][0]) < (float)kPairHi);
 #pragma unroll
       for (int q = 1; q < 4; ++q) far = far || !(fabsf(dx[s][q]) < (float)kPairHi);
     }
