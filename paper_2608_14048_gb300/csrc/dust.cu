@@ -63,6 +63,79 @@ __device__ __forceinline__ void dust_flux(const R* wl, const R* wr, R* f) {
     f[q] = R(0.5) * (ul[q] * vnl + ur[q] * vnr) - R(0.5) * sp * (ur[q] - ul[q]);
 }
 
+// The same in FP32, and the PPM and PPM5 face states, with every rounding written
+// out: the two cells of a face compute its flux each for itself, and what the compiler
+// fuses in one place and not in the other would give a face two fluxes (what leaves
+// one cell would not be what enters the next).
+template <int D>
+__device__ __forceinline__ void dust_flux(const float* wl, const float* wr, float* f) {
+  const float vl = wl[1 + D], vr = wr[1 + D];
+  const float hs = -0.5f * fmaxf(fabsf(vl), fabsf(vr));
+  float ml[3], mr[3];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    ml[q] = __fmul_rn(wl[0], wl[1 + q]);
+    mr[q] = __fmul_rn(wr[0], wr[1 + q]);
+  }
+  f[0] = __fmaf_rn(0.5f, __fadd_rn(ml[D], mr[D]), __fmul_rn(hs, __fsub_rn(wr[0], wl[0])));
+#pragma unroll
+  for (int q = 0; q < 3; ++q)
+    f[1 + q] = __fmaf_rn(0.5f, __fmaf_rn(ml[q], vl, __fmul_rn(mr[q], vr)),
+                         __fmul_rn(hs, __fsub_rn(mr[q], ml[q])));
+}
+// ppm_iface, ppm5_left, ppm5_right (clipped) and ppm_limit of common.cuh
+__device__ __forceinline__ float dust_iface(const float* s) {
+  const float x = __fadd_rn(s[1], s[2]), y = __fadd_rn(s[0], s[3]);
+  return clip_pair(__fmaf_rn((float)(7.0 / 12.0), x, -__fmul_rn((float)(1.0 / 12.0), y)), s[1], s[2]);
+}
+__device__ __forceinline__ float dust_left(const float* q) {
+  float a = __fmaf_rn(27.0f, q[1], __fmul_rn(-3.0f, q[0]));
+  a = __fmaf_rn(2.0f, q[4], __fmaf_rn(-13.0f, q[3], __fmaf_rn(47.0f, q[2], a)));
+  return clip_pair(__fmul_rn(a, (float)(1.0 / 60.0)), q[1], q[2]);
+}
+__device__ __forceinline__ float dust_right(const float* q) {
+  float a = __fmaf_rn(-13.0f, q[1], __fmul_rn(2.0f, q[0]));
+  a = __fmaf_rn(-3.0f, q[4], __fmaf_rn(27.0f, q[3], __fmaf_rn(47.0f, q[2], a)));
+  return clip_pair(__fmul_rn(a, (float)(1.0 / 60.0)), q[2], q[3]);
+}
+__device__ __forceinline__ void dust_limit(float w, float& l, float& r) {
+  if (__fmul_rn(__fsub_rn(r, w), __fsub_rn(w, l)) <= 0.0f) {
+    l = r = w;
+    return;
+  }
+  const float d = __fsub_rn(r, l), q = __fmul_rn(d, __fmaf_rn(-0.5f, __fadd_rn(l, r), w));
+  const float d2 = __fmul_rn(__fmul_rn(d, d), (float)(1.0 / 6.0));
+  if (q > d2) l = __fmaf_rn(3.0f, w, -__fmul_rn(2.0f, r));
+  else if (-d2 > q) r = __fmaf_rn(3.0f, w, -__fmul_rn(2.0f, l));
+}
+// Face states of one variable, as recon_face.
+template <int RECON>
+__device__ __forceinline__ void dust_states(const float* s, float& wl, float& wr) {
+  if constexpr (RECON < 2) {
+    recon_face<RECON>(s, wl, wr);
+  } else {
+    float l1, r1, l2, r2;
+    if constexpr (RECON == 2) {
+      l1 = dust_iface(s);
+      r1 = l2 = dust_iface(s + 1);
+      r2 = dust_iface(s + 2);
+    } else {
+      l1 = dust_left(s);
+      r1 = dust_right(s);
+      l2 = dust_left(s + 1);
+      r2 = dust_right(s + 1);
+    }
+    dust_limit(s[2], l1, r1);
+    dust_limit(s[3], l2, r2);
+    wl = r1;
+    wr = l2;
+  }
+}
+template <int RECON>
+__device__ __forceinline__ void dust_states(const double* s, double& wl, double& wr) {
+  recon_face<RECON>(s, wl, wr);
+}
+
 // Flux across the D-face between cells w[2] and w[3] of a line of cells.
 template <int RECON, int D, typename R>
 __device__ __forceinline__ void dust_face(const R (*w)[4], R* f) {
@@ -72,7 +145,7 @@ __device__ __forceinline__ void dust_face(const R (*w)[4], R* f) {
     R s[6];
 #pragma unroll
     for (int t = 0; t < 6; ++t) s[t] = w[t][q];
-    recon_face<RECON>(s, wl[q], wr[q]);
+    dust_states<RECON>(s, wl[q], wr[q]);
   }
   dust_flux<D>(wl, wr, f);
 }
@@ -121,10 +194,10 @@ __global__ void __launch_bounds__(256)
 // is computed by both of its cells, cheaper than an exchange (the kernel has no
 // barrier).  128^3, 8 species, PLM: three passes of fluxes
 // 475 us, this one 456 (932 instructions a cell and species, issue rate 88%).
-template <typename R, int RECON>
+template <int RECON>
 __global__ void __launch_bounds__(128)
-    k_dust_div(Layout L, const R* __restrict__ dsrc, R* __restrict__ ddiv, int nd, int kc, R idx1,
-               R idx2, R idx3, R dfloor) {
+    k_dust_div(Layout L, const float* __restrict__ dsrc, float* __restrict__ ddiv, int nd, int kc,
+               float idx1, float idx2, float idx3, float dfloor) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   const int s = (int)(blockIdx.z % (unsigned)nd);
@@ -132,28 +205,28 @@ __global__ void __launch_bounds__(128)
   if (i >= L.n[0] || j >= L.n[1]) return;
   constexpr int RH = recon_reach<RECON>(), RL = RH + 1;
   const long long sz = L.size(), sx = L.sx, sxy = L.sx * L.sy;
-  const R* rho = dsrc + (long long)(4 * s) * sz;
-  R* out = ddiv + (long long)(4 * s) * sz;
-  auto load = [&](long long at, R* w) {
-    R r = rho[at];
+  const float* rho = dsrc + (long long)(4 * s) * sz;
+  float* out = ddiv + (long long)(4 * s) * sz;
+  auto load = [&](long long at, float* w) {
+    float r = rho[at];
     if (r < dfloor) r = dfloor;
-    const R ir = recip(r);
+    const float ir = recip(r);
     w[0] = r;
 #pragma unroll
-    for (int q = 0; q < 3; ++q) w[1 + q] = rho[(long long)(1 + q) * sz + at] * ir;
+    for (int q = 0; q < 3; ++q) w[1 + q] = __fmul_rn(rho[(long long)(1 + q) * sz + at], ir);
   };
   // entries t of a line: cells t - 3 about the current one; outside the
   // reconstruction's reach they stay zero
-  R lz[7][4] = {}, fz[4];
+  float lz[7][4] = {}, fz[4];
   long long c = L.idx(i, j, k0);
 #pragma unroll
   for (int t = 3 - RL; t <= 3 + RH; ++t) load(c + (t - 3) * sxy, lz[t]);
   dust_face<RECON, 2>(lz, fz);
   for (int k = k0; k < k1; ++k, c += sxy) {
     load(c + RL * sxy, lz[3 + RL]);
-    R div[4];
+    float div[4];
     {
-      R l[7][4] = {}, lo[4], hi[4];
+      float l[7][4] = {}, lo[4], hi[4];
 #pragma unroll
       for (int t = 3 - RL; t <= 3 + RL; ++t) {
         if (t != 3) load(c + (t - 3), l[t]);
@@ -165,12 +238,12 @@ __global__ void __launch_bounds__(128)
       dust_face<RECON, 0>(l + 1, hi);
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        div[q] = R(0);
+        div[q] = 0.0f;
         div[q] += (hi[q] - lo[q]) * idx1;
       }
     }
     {
-      R l[7][4] = {}, lo[4], hi[4];
+      float l[7][4] = {}, lo[4], hi[4];
 #pragma unroll
       for (int t = 3 - RL; t <= 3 + RL; ++t) {
         if (t != 3) load(c + (t - 3) * sx, l[t]);
@@ -183,7 +256,7 @@ __global__ void __launch_bounds__(128)
 #pragma unroll
       for (int q = 0; q < 4; ++q) div[q] += (hi[q] - lo[q]) * idx2;
     }
-    R hi[4];
+    float hi[4];
     dust_face<RECON, 2>(lz + 1, hi);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -201,8 +274,10 @@ __global__ void __launch_bounds__(128)
 // The same for FP32 and PLM, the default, on packed pairs (rho, v1), (v2, v3):
 // the pass is bound by the issue rate, and a pair takes one instruction.  515
 // instructions a cell and species, 297 us; the update, which reads a third,
-// 507 / 565 -> 400 / 504 us; the step 2440 -> 1910 us.  The momenta are rounded before their difference, as the scalar
-// text does it (ptxas would fuse a packed product into it).
+// 507 / 565 -> 400 / 504 us; the step 2440 -> 1910 us.  The momenta are rounded before
+// their difference and the velocities before their slopes, in both cells of a face
+// alike (ptxas would fuse a packed product into a packed sum; nzero, -0, makes it a
+// multiply-add, which it leaves alone, with the product's own rounding).
 template <int D>
 __device__ __forceinline__ void dust_flux2(const float2* l, const float2* r, float2* f) {
   const float vl[3] = {l[0].y, l[1].x, l[1].y}, vr[3] = {r[0].y, r[1].x, r[1].y};
@@ -223,7 +298,7 @@ __device__ __forceinline__ void dust_flux2(const float2* l, const float2* r, flo
 
 __global__ void __launch_bounds__(128)
     k_dust_div_plm2(Layout L, const float* __restrict__ dsrc, float* __restrict__ ddiv, int nd,
-                    int kc, float idx1, float idx2, float idx3, float dfloor) {
+                    int kc, float idx1, float idx2, float idx3, float dfloor, float nzero) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   const int s = (int)(blockIdx.z % (unsigned)nd);
@@ -239,8 +314,8 @@ __global__ void __launch_bounds__(128)
     float r = p0[at];
     if (r < dfloor) r = dfloor;
     const float ir = recip(r);
-    w[0] = make_float2(r, p1[at] * ir);
-    w[1] = make_float2(p2[at], p3[at]) * splat(ir);
+    w[0] = make_float2(r, __fmul_rn(p1[at], ir));
+    w[1] = fma2(make_float2(p2[at], p3[at]), splat(ir), splat(nzero));
   };
   // half slopes of the middle cell of three
   auto half = [](const float2* a, const float2* b, const float2* c, float2* h) {
@@ -835,15 +910,15 @@ static void stage_dust(aeth_ctx* c, int b, int src, int stage) {
     int kc = 16;
     while (kc > 4 && ctas(kc) < 8LL * c->num_sms) kc /= 2;
     while ((long long)ceil_div(L.n[2], kc) * nd > 65535) kc *= 2;   // grid limit
-    auto divergence = [&](auto kernel) {
+    auto divergence = [&](auto kernel, auto... more) {
       const dim3 grd(ceil_div(L.n[0], 32), ceil_div(L.n[1], 4), ceil_div(L.n[2], kc) * nd);
-      kernel<<<grd, dim3(32, 4), 0, s>>>(L, P.dust[src], P.dflux, nd, kc, i1, i2, i3, dfl);
+      kernel<<<grd, dim3(32, 4), 0, s>>>(L, P.dust[src], P.dflux, nd, kc, i1, i2, i3, dfl, more...);
     };
     switch (c->cfg.recon) {
-      case AETH_RECON_DONOR: divergence(k_dust_div<R, 0>); break;
-      case AETH_RECON_PLM: divergence(k_dust_div_plm2); break;
-      case AETH_RECON_PPM5: divergence(k_dust_div<R, 3>); break;
-      default: divergence(k_dust_div<R, 2>);
+      case AETH_RECON_DONOR: divergence(k_dust_div<0>); break;
+      case AETH_RECON_PLM: divergence(k_dust_div_plm2, -0.0f); break;
+      case AETH_RECON_PPM5: divergence(k_dust_div<3>); break;
+      default: divergence(k_dust_div<2>);
     }
     c->n_launch += 1;
   } else {
