@@ -399,9 +399,11 @@ struct DustUpd {
   R dfloor;
 };
 
-// Bounds of the densities, momenta and implicit weights that the FP32 pairs take:
-// the low halves of their products stay above the smallest normal number
-// (what overflows shows in the sum of the drift energies).
+// Bounds of the densities and implicit weights that the FP32 pairs take: the low halves
+// of their products stay above the smallest normal number.  Momenta have the upper
+// bound only (what overflows shows in the sum of the drift energies): a product below
+// 2^-78 loses low bits to the flush of denormals, an absolute error of 2^-126, which
+// reaches the FP32 rounding of results below about 2^-102 (2e-31).
 constexpr double kPairLo = 1e-10, kPairHi = 1e10;
 
 // The implicit drag of one cell in FP32 pairs: X = (gx, dx) -> (gy, dy), the
