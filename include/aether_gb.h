@@ -445,12 +445,16 @@ aeth_status aeth_set_flux_tile(aeth_ctx* ctx, int flux_tx, int kchunk);
 aeth_status aeth_get_flux_tile(aeth_ctx* ctx, int* flux_tx, int* kchunk);
 
 /* Autotuner of the flux pass's tile shape (no counterpart in the paper):
- * times the fused flux pass for z-chunks of 8, 16, 32 and 64 planes per
+ * times the fused flux pass for the default z-chunk, the even divisions of
+ * the tallest block next to it, and chunks of 8, 16, 32 and 64 planes per
  * tile, with the 32-wide and (where built) the 16-wide and band tiles, on
  * the current state, and keeps the fastest (written to *flux_tx and
- * *kchunk, either may be NULL).  NOTE: it ADVANCES the state by 3 steps per
- * candidate (up to 36) with the current device dt; call it on a scratch copy or
- * before loading the real state.  The Python helper Solver.tune_tiles
+ * *kchunk, either may be NULL).  Contexts whose tiles of 8 planes do not
+ * give every SM one are timed with the last four chunks only; their default
+ * (shorter) chunk is the faster one: leave them untuned.  NOTE: it ADVANCES
+ * the state by 3 steps per candidate and one per width (up to 66) with the
+ * current device dt; call it on a scratch copy or before loading the real
+ * state.  The Python helper Solver.tune_tiles
  * keeps each choice in a JSON cache keyed by the block sizes and the
  * configuration. */
 aeth_status aeth_autotune(aeth_ctx* ctx, int* flux_tx, int* kchunk);

@@ -12,6 +12,7 @@ raises at import of the library (no CPU fallback exists).
 from __future__ import annotations
 
 import ctypes as C
+import functools
 import os
 
 import numpy as np
@@ -407,9 +408,10 @@ def aeth_profile_read(ctx):
 
 
 def aeth_autotune(ctx):
-    """Time the flux pass's tile candidates (widths 32 / 16 / band tiles,
-    z-chunks 8..64) on the current state (which it advances) and keep the
-    fastest; returns (flux_tx, kchunk), flux_tx 0 for band tiles."""
+    """Time the flux pass's tile candidates (widths 32 / 16 / band tiles; the
+    default z-chunk, its neighbours and 8..64) on the current state (which it
+    advances) and keep the fastest; returns (flux_tx, kchunk), flux_tx 0 for
+    band tiles."""
     tx, kc = C.c_int(0), C.c_int(0)
     _check(ctx, load_library().aeth_autotune(ctx, C.byref(tx), C.byref(kc)))
     return tx.value, kc.value
@@ -425,9 +427,23 @@ def aeth_get_flux_tile(ctx):
     return tx.value, kc.value
 
 
+@functools.lru_cache(maxsize=1)
+def tile_kernels():
+    """Digest of the flux pass's sources and of the tuner's candidates: a shape
+    timed on other kernels is no choice for these."""
+    import hashlib
+    d = os.path.join(os.path.dirname(os.path.abspath(__file__)), "csrc")
+    h = hashlib.sha256()
+    for f in ("flux3.cuh", "riemann2.cuh", "pair.cuh", "stage.cuh", "common.cuh", "aux.cu", "runtime.cu"):
+        with open(os.path.join(d, f), "rb") as s:
+            h.update(s.read())
+    return h.hexdigest()[:16]
+
+
 def tile_cache_key(cfg, descs, device=""):
     """Key of a tuned flux-tile shape: the configuration fields that change
-    the flux pass, the block sizes (as a multiset) and the device name."""
+    the flux pass, the block sizes (as a multiset), the device name and the
+    kernels."""
     import hashlib
     import json
     blocks = {}
@@ -437,7 +453,7 @@ def tile_cache_key(cfg, descs, device=""):
     body = {"eos": cfg.eos, "precision": cfg.precision, "recon": cfg.recon,
             "riemann": cfg.riemann, "integrator": cfg.integrator, "path": cfg.path,
             "dual": cfg.dual_energy, "n_dust": cfg.n_dust,
-            "blocks": sorted(blocks.items()), "device": device}
+            "blocks": sorted(blocks.items()), "device": device, "kernels": tile_kernels()}
     return hashlib.sha256(json.dumps(body, sort_keys=True).encode()).hexdigest()[:24], body
 
 

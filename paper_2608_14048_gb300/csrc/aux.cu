@@ -177,7 +177,7 @@ aeth_status build_geometry(aeth_ctx* c) {
 // 199 (2); hydro 34 x 124 x 42 129 (5), 163 (3); PPM 80^3 382 (10), 445 (6).  Over 60
 // combinations of sizes, reconstructions and closures it is within 9% of the best
 // chunk, the one above up to 28% off.
-static int default_kchunk(const aeth_ctx* c) {
+int default_kchunk(const aeth_ctx* c) {
   int nzmax = 1;
   for (const auto& B : c->blocks) nzmax = std::max(nzmax, B.L.n[2]);
   // FP64: the FP64 pipe of an SM, not a slot, is the unit that runs out, so a

@@ -3,6 +3,7 @@
 #include <cuda.h>
 
 #include <cmath>
+#include <algorithm>
 #include <cstring>
 #include <new>
 
@@ -826,25 +827,48 @@ aeth_status aeth_get_flux_tile(aeth_ctx* c, int* flux_tx, int* kchunk) {
 aeth_status aeth_autotune(aeth_ctx* c, int* tx_out, int* kchunk_out) {
   if (!c) return AETH_ERR_ARG;
   if (!c->finalized) return fail(c, AETH_ERR_STATE, "call aeth_finalize first");
-  // three timed steps per candidate (the state advances, as documented)
+  // a warm-up step per width (its kernel may not be loaded yet), three timed steps
+  // per candidate (the state advances, as documented)
   const bool prof = c->profile;
   c->profile = true;
   int best_tx = c->flux_tx, best_kc = c->kchunk;
   double best_ms = 1e300;
+  int nzmax = 1;
+  for (const auto& B : c->blocks) nzmax = std::max(nzmax, B.L.n[2]);
+  auto step = [&]() -> aeth_status {
+    const aeth_status s = enqueue_dt(c);
+    return s == AETH_OK ? enqueue_step(c, false) : s;
+  };
   std::vector<int> widths = {32};
   if (tile_shape_tunable(c)) widths.push_back(16);
   if (band_tiles_fit(c)) widths.push_back(0);
   for (int tx : widths) {
-    for (int kc : {8, 16, 32, 64}) {
-      c->flux_tx = tx;
-      c->kchunk = kc;
+    c->flux_tx = tx;
+    // the chunks of a width: its default and the even divisions next to it, then
+    // plain ones (FP64 64^3 PPM: default 2, 8 took 19% longer a step).  Chunks below 8
+    // only where chunks of 8 give every SM a tile: smaller contexts keep the four plain
+    // ones, and are better left untuned (48 x 40 x 32: 11.4 us a launch by
+    // default, 18.9 in chunks of 8).
+    long long tiles8 = 0;
+    for (const auto& B : c->blocks) tiles8 += tiles_of(B.L, PK_FLUX, 8, tx);
+    std::vector<int> chunks;
+    auto add = [&](int kc) {
+      if (kc < 1 || kc > 64 || (kc < 8 && tiles8 < c->num_sms)) return;
+      if (std::find(chunks.begin(), chunks.end(), kc) == chunks.end()) chunks.push_back(kc);
+    };
+    const int own = default_kchunk(c), parts = ceil_div(nzmax + 2, own);
+    for (int q : {parts, parts + 1, parts - 1})
+      if (q >= 1) add(ceil_div(nzmax + 2, q));
+    for (int kc : {8, 16, 32, 64}) add(kc);
+    for (size_t q = 0; q < chunks.size(); ++q) {
+      c->kchunk = chunks[q];
       aeth_status s = build_tables(c);
+      if (s == AETH_OK && q == 0) s = step();
       if (s != AETH_OK) return s;
       c->prof_used = 0;
       c->prof_bytes = 0;
       for (int rep = 0; rep < 3; ++rep) {
-        s = enqueue_dt(c);
-        if (s == AETH_OK) s = enqueue_step(c, false);
+        s = step();
         if (s != AETH_OK) return s;
       }
       double ms = 0;
@@ -854,7 +878,7 @@ aeth_status aeth_autotune(aeth_ctx* c, int* tx_out, int* kchunk_out) {
       if (n > 0 && ms / n < best_ms) {
         best_ms = ms / n;
         best_tx = tx;
-        best_kc = kc;
+        best_kc = chunks[q];
       }
     }
   }

@@ -205,6 +205,7 @@ aeth_status enqueue_dust_store(aeth_ctx* c, int b, int k, double* io);
 aeth_status enqueue_entropy_store(aeth_ctx* c, int b, double* io);
 aeth_status build_geometry(aeth_ctx* c);
 aeth_status build_tables(aeth_ctx* c);
+int default_kchunk(const aeth_ctx* c);   // for c->flux_tx
 
 // Device-side tile -> block lookup (prefix[b] <= t < prefix[b+1]).
 __device__ __forceinline__ int find_block(const int* __restrict__ pre, int nb, int t) {
