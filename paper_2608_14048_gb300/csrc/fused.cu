@@ -691,7 +691,11 @@ __global__ void __launch_bounds__(256) k_fill_b(Src S, int t0, int reg, int nv) 
   // the axis maps in the order z, y, x, each in the block the previous one
   // leads to: a linked side goes on in the neighbouring block (cells n_nb + p
   // below, p - n above), as the fill axis by axis does
-  const BlockPtrs<R>* SB = &B;
+  // (with links by pointers into the table: the address of a kernel parameter
+  // copied all of it to every thread's stack; one block linked to itself, 128^3 565
+  // -> 485 us a step, 64^3 131 -> 97)
+  const BlockPtrs<R>* const home = LINKS ? B.tab + L.self : &B;
+  const BlockPtrs<R>* SB = home;
   bool up[3];
 #pragma unroll
   for (int e = 2; e >= 0; --e) {
@@ -733,7 +737,7 @@ __global__ void __launch_bounds__(256) k_fill_b(Src S, int t0, int reg, int nv) 
   for (int v = 0; v < NVAR; ++v)
     if (v < nv) {
       // face n of an outflow axis is real: not a copy of itself
-      if (v >= 5 && up[v - 5] && SB == &B && src + L.stride(v - 5) == dst) continue;
+      if (v >= 5 && up[v - 5] && SB == home && src + L.stride(v - 5) == dst) continue;
       B.reg[reg][v][dst] = val[v];
     }
   if constexpr (ENT) B.ent[reg][dst] = ent;   // a cell variable like the density
