@@ -370,6 +370,16 @@ __global__ void __launch_bounds__(256, 1)
 // and 4.  Row-major results at part + chunk * MLP_NPARAM.
 constexpr int DW_K = 16;   // rows staged at a time
 
+// s + c += x, the rounding of each addition kept in c.  The bias gradients are plain
+// sums over up to 271 rows of a chunk, whose order alone would cost them digits (b4 at
+// 256 rows, error against FP64 2.5e-7 in one running sum, 5.2e-8 like this): sixteen rows
+// at a time are added so.
+__device__ __forceinline__ void add_kept(float& s, float& c, float x) {
+  const float t = __fadd_rn(s, x), b = __fsub_rn(t, s);
+  c = __fadd_rn(c, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b)));
+  s = t;
+}
+
 __global__ void __launch_bounds__(256, 2)
     k_mlp_dw(const float* __restrict__ X, RowsOut o, int n, int rows, float* __restrict__ part) {
   const long long r0 = (long long)blockIdx.y * rows, r1 = min((long long)n, r0 + rows);
@@ -380,24 +390,30 @@ __global__ void __launch_bounds__(256, 2)
     // layer 1: thread (o, half) takes 7 inputs; layer 4: thread (i, half) 4
     // outputs (3 in the upper half)
     const int c = tid & 127, half = tid >> 7;
-    float g1[7] = {}, gb1 = 0.0f, g4[4] = {}, gb4 = 0.0f;
+    float g1[7] = {}, gb1 = 0.0f, cb1 = 0.0f, g4[4] = {}, gb4 = 0.0f, cb4 = 0.0f;
+    for (long long s0 = r0; s0 < r1; s0 += DW_K) {
+      const long long s1 = min(s0 + DW_K, r1);
+      float t1 = 0.0f, t4 = 0.0f;   // sixteen rows of the biases
 #pragma unroll 4
-    for (long long s = r0; s < r1; ++s) {
-      const float d = o.dz[0][s * 128 + c], a = o.act[2][s * 128 + c];
+      for (long long s = s0; s < s1; ++s) {
+        const float d = o.dz[0][s * 128 + c], a = o.act[2][s * 128 + c];
 #pragma unroll
-      for (int q = 0; q < 7; ++q) g1[q] += d * X[s * MLP_INP + 7 * half + q];
-      gb1 += d;
+        for (int q = 0; q < 7; ++q) g1[q] += d * X[s * MLP_INP + 7 * half + q];
+        t1 += d;
 #pragma unroll
-      for (int q = 0; q < 4; ++q) g4[q] += a * o.dy[s * MLP_OUTP + 4 * half + q];
-      if (tid < MLP_OUT) gb4 += o.dy[s * MLP_OUTP + tid];
+        for (int q = 0; q < 4; ++q) g4[q] += a * o.dy[s * MLP_OUTP + 4 * half + q];
+        if (tid < MLP_OUT) t4 += o.dy[s * MLP_OUTP + tid];
+      }
+      add_kept(gb1, cb1, t1);
+      add_kept(gb4, cb4, t4);
     }
 #pragma unroll
     for (int q = 0; q < 7; ++q) part[c * MLP_IN + 7 * half + q] = g1[q];
-    if (half == 0) part[128 * MLP_IN + c] = gb1;
+    if (half == 0) part[128 * MLP_IN + c] = gb1 + cb1;
 #pragma unroll
     for (int q = 0; q < 4; ++q)
       if (4 * half + q < MLP_OUT) part[OFF4 + (4 * half + q) * 128 + c] = g4[q];
-    if (tid < MLP_OUT) part[OFF4 + MLP_OUT * 128 + tid] = gb4;
+    if (tid < MLP_OUT) part[OFF4 + MLP_OUT * 128 + tid] = gb4 + cb4;
     return;
   }
   const int l = 1 + blockIdx.x;   // gradient of hidden layer l + 1
@@ -406,7 +422,7 @@ __global__ void __launch_bounds__(256, 2)
   __shared__ __align__(16) float sD[2][DW_K][128], sA[2][DW_K][128];
   const int tx = tid & 15, ty = tid >> 4;
   float2 acc[8][4];
-  float gb = 0.0f;
+  float gb = 0.0f, cb = 0.0f;
 #pragma unroll
   for (int p = 0; p < 8; ++p)
 #pragma unroll
@@ -450,8 +466,11 @@ __global__ void __launch_bounds__(256, 2)
         for (int q = 0; q < 4; ++q) fma2(acc[p][q], make_float2(a[p], a[p]), b[q]);
     }
     if (tid < 128) {
+      float t = 0.0f;
 #pragma unroll
-      for (int k = 0; k < DW_K; ++k) gb += sD[buf][k][tid];
+      for (int k = 0; k < DW_K; k += 4)
+        t += (sD[buf][k][tid] + sD[buf][k + 1][tid]) + (sD[buf][k + 2][tid] + sD[buf][k + 3][tid]);
+      add_kept(gb, cb, t);
     }
     __syncthreads();
   }
@@ -464,7 +483,7 @@ __global__ void __launch_bounds__(256, 2)
       out[m * 128 + c] = acc[p][q].x;
       out[m * 128 + c + 1] = acc[p][q].y;
     }
-  if (tid < 128) out[128 * 128 + tid] = gb;
+  if (tid < 128) out[128 * 128 + tid] = gb + cb;
 }
 
 // grad = sum of the chunks' gradients: four groups of chunks a parameter, in
