@@ -80,8 +80,8 @@ constexpr bool iso_solver(int solver) { return solver == 3 || solver == 4; }
 
 // Riemann solver family SOLVER (numbering of k_flux3 below) on one face: on
 // packed pairs in FP32 (all but the isothermal HLLE), else the scalar solvers;
-// a gas without field takes either without its terms.  SPLIT: see riemann2.cuh;
-// set for the z faces of donor-cell states, whose rounding it fixes.
+// a gas without field takes either without its terms.  SPLIT: the rounding of one
+// term of the right side (riemann2.cuh), set for the z faces of donor-cell states.
 template <int SOLVER, bool MHD, bool SPLIT, typename R>
 __device__ __forceinline__ void solve_face(R g, R igm1, const R* wl, const R* wr, R bn, R* fx) {
   if constexpr (sizeof(R) == 4 && SOLVER != 4) {

@@ -88,9 +88,13 @@ struct SidePair {
   }
 };
 
-// HLLD (hlld_s of common.cuh; LD: LHLLD); MHD = false: HLLC / LHLLC.  SPLIT:
-// the right side's normal momentum flux subtracts a rounded bn^2 like the left
-// side's, instead of fusing the product.
+// HLLD (hlld_s of common.cuh; LD: LHLLD); MHD = false: HLLC / LHLLC.  SPLIT decides
+// one rounding of the right side.  The left normal momentum flux subtracts bn^2
+// rounded; the right one does the same with SPLIT, and without it subtracts the
+// unrounded square in one multiply-add.  So without SPLIT the solver is mirror
+// symmetric up to that last bit only.  Both forms are what the scalar solver's compiled
+// text rounded to (SPLIT: z faces of donor states), kept so that results stay
+// comparable bit for bit.
 template <bool LD, bool MHD, bool SPLIT>
 __device__ __forceinline__ void hlld2(float gamma, float igm1, const float2* W, float bn, float* f) {
   const float bn2 = rmul(bn, bn);
@@ -193,7 +197,9 @@ __device__ __forceinline__ void hlld2(float gamma, float igm1, const float2* W, 
 }
 
 // Isothermal HLLD (hlld_iso of common.cuh), g = cs^2.  SPLIT: the right side's
-// induction fluxes are differences of two rounded products.
+// induction fluxes are differences of two rounded products, the left side's (and
+// without SPLIT both) one multiply-add of a rounded product: again the last bit in
+// which the two sides differ.
 template <bool MHD, bool SPLIT>
 __device__ __forceinline__ void hlld_iso2(float g, const float2* W, float bn, float* f) {
   const float bn2 = rmul(bn, bn);
