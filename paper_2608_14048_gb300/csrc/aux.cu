@@ -170,13 +170,13 @@ aeth_status build_geometry(aeth_ctx* c) {
 // (16).  The longest chunk with four tiles an SM, the rule before, took 64, 32
 // and 16 of these.
 // FP32_P64 recovers every staged cell's pressure in FP64, so the FP64 pipe of
-// the SMs bounds the pass, through the warm-up planes too (w 2), and tiles go
-// in waves: a wave costs as many tiles as an SM holds, and the last one never
-// less than four, whose warps the pipe needs to stay busy.  us per step, by
-// this rule and by the one above: PLM 64^3 191 (kc 6), 229 (3); 150 x 20 x 60 158 (4),
-// 199 (2); hydro 34 x 124 x 42 129 (5), 163 (3); PPM 80^3 382 (10), 445 (6).  Over 60
-// combinations of sizes, reconstructions and closures it is within 9% of the best
-// chunk, the one above up to 28% off.
+// the SMs bounds the pass, through the warm-up planes too (w 2; donor cells, with
+// no halo, 0.8), and tiles go in waves: a wave costs as many tiles as an SM
+// holds, and the last one never less than 4.5, whose warps the pipe needs to stay
+// busy.  us per step, by this rule and by the one above: PLM 64^3 191 (kc 6), 229 (3);
+// 150 x 20 x 60 158 (4), 199 (2); hydro 34 x 124 x 42 129 (5), 163 (3); PPM 80^3 382
+// (10), 445 (6).  Over 60 combinations of sizes, reconstructions and closures it is
+// within 7% of the best chunk, the one above up to 28% off.
 int default_kchunk(const aeth_ctx* c) {
   int nzmax = 1;
   for (const auto& B : c->blocks) nzmax = std::max(nzmax, B.L.n[2]);
@@ -190,7 +190,8 @@ int default_kchunk(const aeth_ctx* c) {
   const bool p64 = c->cfg.precision == AETH_FP32_P64 && !is_iso(c);
   const int per_sm = f64 ? 2 : (c->flux_tx ? (ppm ? 4 : 5) : 2);
   const double slots = (double)c->num_sms * per_sm;
-  const double w = f64 ? 0.3 : (ppm || p64 ? 2.0 : 1.0), tail = f64 ? 1.0 : 0.5;
+  const bool donor = c->cfg.recon == AETH_RECON_DONOR;
+  const double w = f64 ? 0.3 : (p64 && donor ? 0.8 : (ppm || p64 ? 2.0 : 1.0)), tail = f64 ? 1.0 : 0.5;
   int best = 1;
   double best_cost = 1e300;
   // the even divisions of the tallest block
@@ -209,10 +210,11 @@ int default_kchunk(const aeth_ctx* c) {
     if (f64 && tiles <= slots) cost = 1.35 * (kc + w);
     if (p64) {
       const long long wave = (long long)c->num_sms * per_sm, rest = tiles % wave;
-      const int last = rest ? std::max(ceil_div(rest, c->num_sms), std::min(4, per_sm)) : 0;
+      const double last =
+          rest ? std::max((double)ceil_div(rest, c->num_sms), std::min(4.5, (double)per_sm)) : 0.0;
       cost = ((double)(tiles / wave) * per_sm + last) * (kc + w);
     }
-    if (cost < best_cost) {
+    if (cost < best_cost || (p64 && cost == best_cost)) {   // of equal ones the shorter
       best_cost = cost;
       best = kc;
     }
