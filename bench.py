@@ -61,7 +61,8 @@ def parse(argv=None):
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--workload", default="turb256", choices=WORKLOADS)
     ap.add_argument("--drag", default="fp64", choices=["fp64", "fp32", "sel"],
-                    help="dust128: drag solve in FP64, FP32, or FP64 only for the stiff species")
+                    help="dust128: drag solve in FP64 (FP32 pairs under FP32 transport), FP32, or "
+                         "the former only for the stiff species")
     ap.add_argument("--no-autotune", action="store_true")
     ap.add_argument("--train-on", default="c2", choices=["c2", "c5"],
                     help="learned512: the network's training states: the 256^3 Mach-2 "

@@ -124,8 +124,11 @@ typedef struct {
                            drag_law = AETH_DRAG_LAW_COEFF the drag
                            coefficients K_k (copied; each > 0) */
   int drag_precision; /* AETH_DRAG_FP64 (default, 0): implicit drag solve in
-                         FP64; AETH_DRAG_FP32: in FP32; AETH_DRAG_SEL64: in
-                         FP64 only for the species whose implicit weight
+                         FP64, under FP32 transport and constant stopping
+                         times in FP32 pairs of about 48 bits (FP64 for cells
+                         outside densities and weights of 1e-10 .. 1e10);
+                         AETH_DRAG_FP32: in FP32; AETH_DRAG_SEL64: in
+                         pairs only for the species whose implicit weight
                          h / t_k (h = the stage's implicit step) exceeds
                          drag_ratio, in FP32 for the others (dust runs
                          only; AETH_FP64 and AETH_FP32 keep their values) */
@@ -156,7 +159,7 @@ typedef struct {
                           4, where the FP32 subtraction's relative error,
                           about 4 ulp x the ratio, stays below 1e-6 */
   double drag_ratio;   /* AETH_DRAG_SEL64: species with h / t_k > drag_ratio
-                          are solved in FP64; <= 0 selects 1 */
+                          are solved in pairs; <= 0 selects 1 */
   int drag_law;        /* AETH_DRAG_LAW_TSTOP (default, 0) or
                           AETH_DRAG_LAW_COEFF; the latter takes a_k =
                           h K_k / rho_k per cell (a species with rho_k <= 0

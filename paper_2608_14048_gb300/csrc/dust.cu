@@ -2,10 +2,10 @@
 //
 // Per stage: ghost fill; the fused hydro-gas flux pass (HLLD at B = 0); the
 // pressureless Rusanov fluxes of every species (FP32: one pass that leaves their
-// divergence; FP64: a flux pass per direction); then one fused kernel that forms the explicit stage combination and solves the
-// implicit drag of every cell in closed form (arrowhead system, O(N) per
-// velocity component) in FP64 by default (aeth_config.drag_precision),
-// whatever the transport precision.
+// divergence; FP64: a flux pass per direction); then one fused kernel that forms
+// the explicit stage combination and solves the implicit drag of every cell in
+// closed form (arrowhead system, O(N) per velocity component), by default
+// (aeth_config.drag_precision) in FP64 or, under FP32 transport, FP32 pairs.
 //
 // The stage combinations run in the working precision.  GB300 executes an FP64
 // operation at 1/64 of the FP32 rate, and the solve's ~215 operations and ~65
@@ -564,8 +564,9 @@ __device__ __noinline__ void drag_far(const float* gx, const float (*dx)[4], int
 // rho_k per cell).  iso: isothermal gas, whose energy slot takes no drag
 // heating.
 // Bounds: five CTAs of 128 threads an SM for the solve in pairs of up to 8 species
-// (102 registers): 128^3, 8 species, step 1909 -> 1897 us against the compiler's own
-// 128 registers; 61 x 100 x 37, 3 species 210 -> 205.  The others keep what they need.
+// (96 registers; the two for 8 species spill about 120 bytes): 128^3, 8 species, step
+// 1909 -> 1897 us against the compiler's own 128 registers; 61 x 100 x 37, 3 species
+// 210 -> 205.  The others keep what they need.
 template <typename DT, int NDMAX>
 constexpr bool upd_five = std::is_same_v<DT, dfloat> && NDMAX <= 8;
 template <typename R, typename DT, int NDMAX, bool SEL = false, bool COEFF = false>
@@ -577,7 +578,7 @@ __global__ void __launch_bounds__(upd_five<DT, NDMAX> ? 128 * AETH_DUST_BZ : 256
   // a_k = h / t_k, 1 / (1 + a_k), w_k = a_k / (1 + a_k) with h = g dt
   __shared__ DT s_ak[NDMAX], s_ia[NDMAX], s_wk[NDMAX];
   __shared__ float f_ak[SEL ? NDMAX : 1], f_ia[SEL ? NDMAX : 1], f_wk[SEL ? NDMAX : 1];
-  __shared__ unsigned s_wide;   // SEL: bit s set = species s in FP64
+  __shared__ unsigned s_wide;   // SEL: bit s set = species s in pairs
   // PAIR: the FP64 solve in FP32 pairs; the FP64 constants stay for the cells
   // outside the pairs' range
   constexpr bool PAIR = std::is_same_v<DT, dfloat>;
@@ -601,7 +602,7 @@ __global__ void __launch_bounds__(upd_five<DT, NDMAX> ? 128 * AETH_DUST_BZ : 256
         s_ia[tid] = dfloat::of(ia);
         s_wk[tid] = dfloat::of(a * ia);
         // a constant of a species that the pairs solve (an uncoupled FP32 species sent
-        // every cell to FP64: 64^3, 4 species 392 us a step, 200 now)
+        // every cell to FP64: 64^3, 4 species 392 us a step, 192 now)
         if ((!SEL || a > (CT)sel_ratio) && !(a > kPairLo && a < kPairHi)) s_far = 1;
       } else {
         s_ak[tid] = a;
@@ -969,7 +970,7 @@ static void stage_dust(aeth_ctx* c, int b, int src, int stage) {
   bool done = false;
   if constexpr (sizeof(R) == 4) {
     if (c->cfg.drag_precision == AETH_DRAG_SEL64) {
-      // per-species precision: FP64 for the species with h / t_k > drag_ratio
+      // per-species precision: pairs for the species with h / t_k > drag_ratio
       if (nd <= 8) launch(k_dust_update<R, dfloat, 8, true>);
       else launch(k_dust_update<R, dfloat, 32, true>);
       done = true;
